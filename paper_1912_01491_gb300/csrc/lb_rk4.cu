@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "lb_internal.h"
+#include "lb_rowsum.cuh"
 
 namespace {
 
@@ -86,9 +87,8 @@ __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __re
       a3 = fmaf(u.w, xu.w, a3);
     }
     for (int64_t n = head + 4 * nv + lane; n < M; n += 32) a0 = fmaf(__ldcs(row + n), __ldg(x32 + n), a0);
-    double t = ((double)a0 + (double)a1) + ((double)a2 + (double)a3);
-    for (int o2 = 16; o2 > 0; o2 >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o2);
-    return t;
+    const float a[4] = {a0, a1, a2, a3};
+    return lb::lane_sum(a);
   } else {
     // BF16: lane k reads four values (8 bytes) of A at element head + 4k
     // (head up to the first 8-byte boundary) and the matching float4 of the
@@ -131,9 +131,8 @@ __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __re
     }
     for (int64_t n = head + 4 * nv + lane; n < M; n += 32)
       a0 = fmaf(bf16_bits_to_float(__ldcs(reinterpret_cast<const unsigned short*>(row + n))), __ldg(x32 + n), a0);
-    double t = ((double)a0 + (double)a1) + ((double)a2 + (double)a3);
-    for (int o2 = 16; o2 > 0; o2 >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o2);
-    return t * (double)__ldg(scale + s);
+    const float a[4] = {a0, a1, a2, a3};
+    return __dmul_rn(lb::lane_sum(a), (double)__ldg(scale + s));
   }
 }
 
@@ -148,19 +147,13 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   if (s >= M) return;
   const double y = row_dot<PREC>(M, s, Ap, scale, x, x32, xstride, lane);
   if (lane != 0) return;
-  const double k = y + Keff[s];
+  const double k = y + Keff[s], vs = v[s];
   double nx;
-  if (STAGE == 1) {
-    acc[s] = k;
-    nx = v[s] + 0.5 * h * k;
-  } else if (STAGE == 2) {
-    acc[s] += 2.0 * k;
-    nx = v[s] + 0.5 * h * k;
-  } else if (STAGE == 3) {
-    acc[s] += 2.0 * k;
-    nx = v[s] + h * k;
+  if (STAGE < 4) {
+    acc[s] = STAGE == 1 ? k : fma(2.0, k, acc[s]);
+    nx = fma(h, k, vs);  // h: the stage's step, dt / 2, dt / 2, dt
   } else {
-    nx = v[s] + (h / 6.0) * (acc[s] + k);
+    nx = fma(h, acc[s] + k, vs);  // h: dt / 6
     v[s] = nx;
   }
   xn[s] = nx;
@@ -185,7 +178,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   double t = 0.0;
   if (PREC == LB_FP32) {
     const float* __restrict__ r = static_cast<const float*>(Ap) + s * M;
-    for (int64_t n = lane; n < M; n += 32) t = fma(__ldcs(r64 + n) - (double)__ldcs(r + n), v[n], t);
+    for (int64_t n = lane; n < M; n += 32) t = fma(__ldcs(r64 + n) - lb::widen(__ldcs(r + n)), v[n], t);
   } else {
     // sum_n A64_sn v_n - r_s sum_n q_sn v_n: two FP64 dot products (the
     // difference is formed once per row, not per entry)
@@ -194,10 +187,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     for (int64_t n = lane; n < M; n += 32) {
       const double vn = v[n];
       t = fma(__ldcs(r64 + n), vn, t);
-      tq = fma((double)bf16_bits_to_float(__ldcs(reinterpret_cast<const unsigned short*>(r + n))), vn, tq);
+      tq = fma(lb::widen(bf16_bits_to_float(__ldcs(reinterpret_cast<const unsigned short*>(r + n)))), vn, tq);
     }
     for (int o = 16; o > 0; o >>= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
-    if (lane == 0) t -= (double)scale[s] * tq;  // once, before the lane sum below
+    if (lane == 0) t = fma(-(double)scale[s], tq, t);  // once, before the lane sum below
   }
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) Keff[s] = K[s] + t;
@@ -772,10 +765,10 @@ cudaError_t run_steps(int64_t M, const void* Ap, const float* scale, const doubl
       k_correction<PREC><<<grid, bs, 0, st>>>(M, A64, Ap, scale, v, K, w.Keff);
       lbi::note_launch(1);
     }
-    k_stage<PREC, 1><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
-    k_stage<PREC, 2><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt);
+    k_stage<PREC, 1><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, 0.5 * dt);
+    k_stage<PREC, 2><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, 0.5 * dt);
     k_stage<PREC, 3><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
-    k_stage<PREC, 4><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt);
+    k_stage<PREC, 4><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt / 6.0);
     lbi::note_launch(4);
     if (snaps && snap_every > 0 && (t + 1) % snap_every == 0) {
       e = cudaMemcpyAsync(snaps + ((t + 1) / snap_every - 1) * M, v, sizeof(double) * M,
