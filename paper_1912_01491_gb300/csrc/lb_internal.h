@@ -102,7 +102,15 @@ size_t rk4_workspace_bytes(int64_t M);
 cudaError_t rk4_dense(int64_t M, int precision, const void* Ap, const float* scale,
                       const double* A64, int correct_every, const double* K, double* v,
                       double dt, int64_t nsteps, double* snaps, int64_t snap_every,
-                      void* work, cudaStream_t st);
+                      void* work, cudaStream_t st, bool one_launch = true);
+// All steps in one cooperative launch (lb_rk4_persist.cu), bit-identical to
+// the stage launches: whether the size is in its range, and the launch
+// (*done = false: not taken, nothing enqueued).  ll: 32 M bytes, keff: M
+// doubles, err: one int of device scratch.
+bool rk4_persist_applies(int64_t M, int precision);
+cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* scale, const double* A64,
+                        int correct_every, const double* K, double* v, double dt, int64_t nsteps, double* snaps,
+                        int64_t snap_every, double* keff, void* ll, int* err, cudaStream_t st, bool* done);
 
 // batched form (lb_batch.cu): one realization of the cluster-persistent RK4
 struct BatchItem {

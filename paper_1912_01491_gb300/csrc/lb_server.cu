@@ -228,7 +228,7 @@ cudaError_t enqueue_stream_rk4(lb_server* s, Req* r) {
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(s->cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
     const cudaError_t ec = lbi::rk4_dense(M, prec, Ap, r->scale, A64, corr, r->K, r->v, r->q.dt, chunk, nullptr, 0,
-                                          r->work, s->cap);
+                                          r->work, s->cap, false);
     e = cudaStreamEndCapture(s->cap, &g);
     if (ec != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
@@ -245,7 +245,7 @@ cudaError_t enqueue_stream_rk4(lb_server* s, Req* r) {
   }
   if (tail > 0)
     if ((e = lbi::rk4_dense(M, prec, Ap, r->scale, A64, corr, r->K, r->v, r->q.dt, tail, nullptr, 0, r->work,
-                            r->st)) != cudaSuccess)
+                            r->st, false)) != cudaSuccess)
       return e;
   return cudaSuccess;
 }
