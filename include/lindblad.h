@@ -112,14 +112,13 @@ int lb_basis_dims(const lb_basis_t *b, int *N, int64_t *M, int64_t *P);
 int lb_basis_label(const lb_basis_t *b, int64_t i, char *type, int *j, int *k);
 
 /* Number of canonical nonzero triples (m <= n <= s) of f (which = LB_F) or
- * d (LB_D) of the basis, counted on the GPU by kernel (a) without storing
- * them.  Synchronous (default stream). */
+ * d (LB_D) of the basis, in closed form. */
 int lb_structure_count(const lb_basis_t *b, int which, int64_t *nnz);
 
 /* Kernel (a): enumerate the canonical nonzero triples, sorted
  * lexicographically by (m, n, s), into caller DEVICE buffers idx3 (3*nnz
- * int32) and val (nnz doubles) by a count pass, an exclusive scan and a fill
- * pass.  capacity is the buffer length in triples; *nnz always receives the
+ * int32) and val (nnz doubles); the place of every row is known in closed
+ * form.  capacity is the buffer length in triples; *nnz always receives the
  * count, and LB_EINVAL is returned (buffers untouched) if capacity < nnz.
  * Synchronous with respect to `stream`. */
 int lb_structure_export(const lb_basis_t *b, int which, int32_t *idx3, double *val,
@@ -132,23 +131,13 @@ int lb_structure_export(const lb_basis_t *b, int which, int32_t *idx3, double *v
  * cudaFree synchronizes the whole device), and real-time or embedded callers
  * that reserve all memory at start-up.  Arguments, outputs, ordering and
  * error behaviour are those of lb_structure_export; the caller passes the
- * basis and the output buffers.  The scratch (per-m counts and their scan)
- * is a file-scope device array of 2 x 65536 int64 (1 MiB) that every GPU
- * loading this library holds until the process exits; the entry point calls
- * no cudaMalloc, cudaFree or allocating library routine.
+ * basis and the output buffers, and no scratch is needed; the entry point
+ * calls no cudaMalloc, cudaFree or allocating library routine, and calls on
+ * several streams and threads do not share anything.
  *   - Limit: M <= 65535 (N <= 256); a larger basis returns LB_EINVAL with a
  *     message naming the limit, and nothing is launched.
- *   - Set-up: every call looks up the array's device address on the current
- *     device with cudaGetSymbolAddress (nothing is cached, so the call stays
- *     valid after a cudaDeviceReset or a recreated context); the first call
- *     on a device loads the module there, so make it before any stream
- *     capture begins.
- *   - Sharing: all calls on a device use the same array, which keeps the last
- *     call's contents (every word a call reads is written earlier in the same
- *     call, so nothing needs clearing).  The call returns after its fill has
- *     finished on `stream`; calls whose GPU work overlaps (from several host
- *     threads at once, on any streams) race on the array and give wrong
- *     results. */
+ *   - Set-up: the first call on a device loads the module there, so make it
+ *     before any stream capture begins. */
 int lb_structure_export_noalloc(const lb_basis_t *b, int which, int32_t *idx3, double *val,
                                 int64_t capacity, int64_t *nnz, void *stream);
 

@@ -181,36 +181,11 @@ int lb_basis_label(const lb_basis_t* b, int64_t i, char* type, int* j, int* k) {
   return LB_OK;
 }
 
-}  // extern "C"
-
-namespace {
-
-// count per m -> exclusive scan; offsets has M+1 entries, offsets[M] = total.
-int count_and_scan(const lb_basis_t* b, int which, DevBuf& offsets, int64_t* total, cudaStream_t st) {
-  const int64_t M = b->M;
-  int rc;
-  DevBuf per;
-  if ((rc = alloc_or_enomem(per, sizeof(int64_t) * (M + 1), "structure counts")) != LB_OK) return rc;
-  if ((rc = alloc_or_enomem(offsets, sizeof(int64_t) * (M + 1), "structure offsets")) != LB_OK) return rc;
-  LB_TRY_CUDA(cudaMemsetAsync(per.as<int64_t>() + M, 0, sizeof(int64_t), st), "structure counts");
-  LB_TRY_CUDA(lbi::structure_count(b->view(), which, per.as<int64_t>(), st), "kernel (a) count");
-  LB_TRY_CUDA(lbi::exclusive_scan(per.as<int64_t>(), offsets.as<int64_t>(), M, st), "scan");
-  LB_TRY_CUDA(cudaMemcpyAsync(total, offsets.as<int64_t>() + M, sizeof(int64_t),
-                              cudaMemcpyDeviceToHost, st),
-              "structure total");
-  LB_TRY_CUDA(cudaStreamSynchronize(st), "kernel (a)");
-  return LB_OK;
-}
-
-}  // namespace
-
-extern "C" {
-
 int lb_structure_count(const lb_basis_t* b, int which, int64_t* nnz) {
   LB_REQUIRE(b != nullptr && nnz != nullptr, "lb_structure_count: NULL argument");
   LB_REQUIRE(which == LB_F || which == LB_D, "lb_structure_count: which = %d", which);
-  DevBuf off;
-  return count_and_scan(b, which, off, nnz, nullptr);
+  *nnz = lbi::structure_total(b->N, which);
+  return LB_OK;
 }
 
 int lb_structure_export(const lb_basis_t* b, int which, int32_t* idx3, double* val, int64_t capacity,
@@ -218,17 +193,12 @@ int lb_structure_export(const lb_basis_t* b, int which, int32_t* idx3, double* v
   LB_REQUIRE(b != nullptr && nnz != nullptr, "lb_structure_export: NULL argument");
   LB_REQUIRE(which == LB_F || which == LB_D, "lb_structure_export: which = %d", which);
   LB_REQUIRE(b->M <= 0x7fffffffLL, "lb_structure_export: M too large for int32 indices");
-  DevBuf off;
-  int64_t total = 0;
-  int rc = count_and_scan(b, which, off, &total, S(stream));
-  if (rc != LB_OK) return rc;
+  const int64_t total = lbi::structure_total(b->N, which);
   *nnz = total;
   LB_REQUIRE(idx3 != nullptr && val != nullptr, "lb_structure_export: NULL output buffer");
   LB_REQUIRE(capacity >= total, "lb_structure_export: capacity %lld < %lld triples",
              (long long)capacity, (long long)total);
-  LB_TRY_CUDA(lbi::structure_fill(b->view(), which, off.as<int64_t>(), idx3, val, S(stream)),
-              "kernel (a) fill");
-  // offsets are freed at scope exit: wait for the fill that reads them
+  LB_TRY_CUDA(lbi::structure_fill(b->view(), which, idx3, val, S(stream)), "kernel (a) fill");
   LB_TRY_CUDA(cudaStreamSynchronize(S(stream)), "kernel (a) fill");
   return LB_OK;
 }

@@ -4,10 +4,7 @@
 // Eq. (rho).
 //
 // Canonical lists hold each unordered triple once as m <= n <= s, sorted by
-// (m, n, s).  Row m's partners n come in increasing index order and for each
-// the third indices s >= n in increasing order, so a count pass, an
-// exclusive scan over m and a fill pass give the sorted list without any
-// sort.  The nonzero triples fall into three classes:
+// (m, n, s).  The nonzero triples fall into three classes:
 //   * three pair elements whose edges form a triangle a-b-c: for given
 //     types of two of them the type of the third is fixed by parity (f: odd
 //     number of J's, d: even);
@@ -16,6 +13,8 @@
 //     for l >= max(a,1) except (a,b,l) = (0,1,1);
 //   * d(D_l, D_l, D_r) for r >= l except l = r = 1 (canonical form of the
 //     "two smallest equal" rule).
+// The number of triples of a row m and of all rows before it are polynomials
+// in the row's vertices, so one pass writes the list: no count, no scan.
 #include "lb_internal.h"
 
 namespace {
@@ -57,133 +56,161 @@ __global__ void k_tables(int N, int32_t* pair_ab, double* tab) {
   }
 }
 
-// One warp per row m.  The candidates of a row are laid out as a sequence of
-// slots whose (n, s) order is the canonical order; the warp takes 32 slots at
-// a time, each lane evaluates one, and a ballot gives each nonzero its place,
-// so the output of a row is written in order by consecutive lanes.
-//
-// Pair row m = (k, a, b).  For each partner type tn >= k (tn < k gives n < m)
-// the partners are the 2N-3 edges that share a vertex with (a,b) or equal it,
-// in lexicographic order:
-//   e <  2a           : (e/2, a) for even e, (e/2, b) for odd e
-//   2a <= e < a+N-1   : (a, e-a+1)           -- holds (a,b) itself at e = a+b-1
-//   a+N-1 <= e < N+b-2: (e-N+2, b)
-//   N+b-2 <= e < 2N-3 : (b, e-N+3)
-// The slot of (a,b) itself is replaced by the run of D_l it pairs with:
-// f(S_ab, J_ab, D_l) for max(a,1) <= l <= b when tn != k, d(X_ab, X_ab, D_l)
-// for max(a,1) <= l < N when tn == k (the zero at (a,b,l) = (0,1,1) is
-// dropped by the value test).  With tn == k the row starts at (a,b).
-// A shared-vertex partner fixes the third edge and, by parity, its type; the
-// triple is canonical when s >= n.
-//
-// Diagonal row m = D_l (d only): d(D_l, D_l, D_r) for r >= l; the zero at
-// l = r = 1 is dropped by the value test.
-struct PairPlan {
-  int pab;    // slot of the edge (a,b): a + b - 1
-  int first;  // first slot of the row
-  int lo, nl; // D run l = lo .. lo + nl - 1
-  int total;  // slots: 2N-4 edges + nl
-};
+// ------------------------------------------------ places of the rows
+// tri(n) = 1 + .. + n, tet(n) = tri(1) + .. + tri(n), sqr(n) = 1 + 4 + .. + n^2.
+LB_HD int64_t tri(int64_t n) { return n * (n + 1) / 2; }
+LB_HD int64_t tet(int64_t n) { return n * (n + 1) * (n + 2) / 6; }
+LB_HD int64_t sqr(int64_t n) { return n * (n + 1) * (2 * n + 1) / 6; }
 
-__device__ __forceinline__ PairPlan pair_plan(int N, const Elem& em, int tn, int which) {
-  PairPlan p;
-  p.pab = em.a + em.b - 1;
-  p.first = tn == em.kind ? p.pab : 0;
-  p.lo = imax(em.a, 1);
-  if (which == LB_F) p.nl = tn != em.kind ? em.b - p.lo + 1 : 0;
-  else p.nl = tn == em.kind ? N - p.lo : 0;
-  p.total = 2 * N - 4 + p.nl;
-  return p;
-}
-
-__device__ __forceinline__ void edge_of_slot(int N, int a, int b, int e, int& u, int& v) {
-  if (e < 2 * a) {
-    u = e >> 1;
-    v = (e & 1) ? b : a;
-  } else if (e < a + N - 1) {
-    u = a;
-    v = e - a + 1;
-  } else if (e < N + b - 2) {
-    u = e - N + 2;
-    v = b;
-  } else {
-    u = b;
-    v = e - N + 3;
+// Canonical triples of the S_ab rows before (a, b), of the J_ab rows before
+// (a, b), and of the D_l rows before l, with lo = max(a, 1) and e = 1 on the
+// edge (0, 1).  A row holds
+//   f: S  2 (N-1-b) + (b-a-1) triangles and b - lo + 1 D_l;  J  N-1-b triangles
+//   d: S  (N-1-b) + (N-2) triangles and N - lo - e D_l;  J  N - lo - e D_l;
+//      D  N - l - [l = 1].
+// (a, b) = (N-1, N) and l = N give the totals.
+LB_HD int64_t rows_s(int64_t N, int which, int64_t a, int64_t b) {
+  const int64_t n = N - 1, lo = a > 1 ? a : 1, in = b - a - 1;
+  if (which == LB_F) {
+    const int64_t before = a == 0 ? 0 : n * (2 * N - 3) + 2 * (sqr(N - 2) - sqr(n - a));
+    return before + in * (2 * N - 2 - a - lo);
   }
-}
-
-// Evaluate slot j of a pair row: (n, s, value); false when the slot holds no
-// canonical triple.
-__device__ __forceinline__ bool pair_slot(const BasisView& B, const Elem& em, int tn, int which,
-                                          const PairPlan& p, int j, int64_t& n, int64_t& s, double& val) {
-  const int N = B.N;
-  double f, d;
-  if (j >= p.pab && j < p.pab + p.nl) {
-    const int l = p.lo + (j - p.pab);
-    n = (int64_t)tn * B.P + pair_index(N, em.a, em.b);
-    s = d_index(B, l);
-    fd_value(B, em, make_pair(tn, em.a, em.b), make_d(l), f, d);
-  } else {
-    int u, v;
-    edge_of_slot(N, em.a, em.b, j < p.pab ? j : j - p.nl + 1, u, v);
-    n = (int64_t)tn * B.P + pair_index(N, u, v);
-    const Elem en = make_pair(tn, u, v);
-    int lo, hi;
-    third_edge(em, en, common_vertex(em, en), lo, hi);
-    const int t3 = which == LB_F ? (1 ^ em.kind ^ tn) : (em.kind ^ tn);
-    s = (int64_t)t3 * B.P + pair_index(N, lo, hi);
-    if (s < n) return false;
-    fd_value(B, em, en, make_pair(t3, lo, hi), f, d);
+  int64_t before = 0;
+  if (a > 0) {
+    const int64_t k = a - 1;  // rows a' = 1 .. k, each 3n^2 - 4n a' + a'^2 - tri(n) + tri(a')
+    before = n * (3 * n - 1) - tri(n) - 1 + k * (3 * n * n - tri(n)) - 4 * n * tri(k) + sqr(k) + tet(k);
   }
-  val = which == LB_F ? f : d;
-  return val != 0.0;
+  return before + in * (3 * n - lo) - (tri(b - 1) - tri(a)) - (a == 0 && b > 1 ? 1 : 0);
+}
+LB_HD int64_t rows_j(int64_t N, int which, int64_t a, int64_t b) {
+  const int64_t n = N - 1, lo = a > 1 ? a : 1;
+  if (which == LB_F) return tet(N - 2) - tet(N - 2 - a) + tri(N - 2 - a) - tri(n - b);
+  const int64_t before = a == 0 ? 0 : n * n - 1 + 2 * (tet(N - 2) - tet(n - a));
+  return before + (b - a - 1) * (N - lo) - (a == 0 && b > 1 ? 1 : 0);
+}
+LB_HD int64_t rows_d(int64_t N, int which, int64_t l) {
+  return which == LB_F ? 0 : tri(N - 1) - tri(N - l) - (l > 1 ? 1 : 0);
 }
 
-// FILL = false: per_m[m] = number of nonzero canonical triples of row m.
-// FILL = true : write row m's triples from offset off[m].
-template <bool FILL>
-__global__ void __launch_bounds__(256) k_rows(BasisView B, int which, int64_t* per_m, const int64_t* off,
-                                              int32_t* idx, double* val) {
+// One warp per row m: lane by lane the row's triples in canonical order, a
+// run of partners n for each class (below, w is the third vertex of a
+// triangle; every triangle's value is 1/sqrt2 up to the stated sign):
+//   f, S_ab: n = S_aw (w > b), S_wb (a < w < b), S_bw (w > b) with the J of
+//            the third edge; then n = J_ab with D_l
+//   f, J_ab: n = J_aw, s = J_bw, w > b
+//   d, S_ab: n = S_ab with D_l; n = S_aw, s = S_bw, w > b; then, w ascending,
+//            the J of the edges to a and to b (minus for a < w < b)
+//   d, J_ab: n = J_ab with D_l
+//   d, D_l:  n = D_l, s = D_r, r >= l
+// Bound by the stores: 20 bytes a triple.  The three indices of 32 triples are
+// 96 consecutive words, which the lanes exchange and write as three runs.  At
+// N = 200 (1.7e7 triples of f and d, both calls) 0.66 ms with a count pass over all
+// candidate partners, a scan and a fill pass, 0.135 ms so (2.5 TB/s).
+__global__ void __launch_bounds__(256) k_rows(BasisView B, int which, int32_t* __restrict__ idx,
+                                              double* __restrict__ val) {
   const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
   const int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (m >= B.M) return;  // whole warps leave together
   const Elem em = decode(B, m);
-  const int N = B.N;
-  int64_t pos = FILL ? off[m] : 0;
-  auto take = [&](bool nz, int64_t n, int64_t s, double v) {
-    const unsigned bal = __ballot_sync(0xffffffffu, nz);
-    if (FILL && nz) {
-      const int64_t o = pos + __popc(bal & below);
-      idx[3 * o] = (int32_t)m;
-      idx[3 * o + 1] = (int32_t)n;
-      idx[3 * o + 2] = (int32_t)s;
-      val[o] = v;
-    }
-    pos += __popc(bal);
+  const int N = B.N, a = em.a, b = em.b, k = em.kind;
+  const int32_t P = (int32_t)B.P;
+  const double c = 2.0 * kInv2Sqrt2;
+  auto edge = [&](int u, int v) {  // pair index (int32: M is)
+    const int x = imin(u, v), y = imax(u, v);
+    return (int32_t)((uint32_t)x * (uint32_t)(2 * N - x - 1) / 2u) + (y - x - 1);
   };
-  if (em.kind == kD) {
+  int64_t off = 0;
+  int cnt = 0, n1 = 0, n2 = 0, lo = 0;
+  const int up = N - 1 - b;  // vertices above b
+  if (k == kD) {
     if (which == LB_D) {
-      const int l = em.a;
-      for (int r0 = l; r0 < N; r0 += 32) {
-        const int r = r0 + lane;
-        const double v = r < N ? 2.0 * trace_ddd(B, l, l, r) : 0.0;
-        take(v != 0.0, m, d_index(B, r < N ? r : l), v);
-      }
+      lo = a == 1 ? 2 : a;
+      cnt = N - lo;
+      off = rows_s(N, which, N - 1, N) + rows_j(N, which, N - 1, N) + rows_d(N, which, a);
     }
   } else {
-    for (int tn = em.kind; tn <= kJ; ++tn) {
-      const PairPlan p = pair_plan(N, em, tn, which);
-      for (int j0 = p.first; j0 < p.total; j0 += 32) {
-        const int j = j0 + lane;
-        int64_t n = 0, s = 0;
-        double v = 0.0;
-        const bool nz = j < p.total && pair_slot(B, em, tn, which, p, j, n, s, v);
-        take(nz, n, s, v);
+    lo = imax(a, 1);
+    if (which == LB_F) {
+      if (k == kS) {
+        n1 = up;
+        n2 = up + b - a - 1;
+        cnt = n2 + up + b - lo + 1;
+        off = rows_s(N, which, a, b);
+      } else {
+        cnt = up;
+        off = rows_s(N, which, N - 1, N) + rows_j(N, which, a, b);
+      }
+    } else {
+      if (a == 0 && b == 1) lo = 2;
+      n1 = N - lo;
+      if (k == kS) {
+        n2 = n1 + up;
+        cnt = n2 + N - 2;
+        off = rows_s(N, which, a, b);
+      } else {
+        cnt = n1;
+        off = rows_s(N, which, N - 1, N) + rows_j(N, which, a, b);
       }
     }
   }
-  if (!FILL && lane == 0) per_m[m] = pos;
+  const int32_t eab = k == kD ? 0 : edge(a, b);
+  for (int e0 = 0; e0 < cnt; e0 += 32) {
+    const int e = e0 + lane;
+    int32_t n = (int32_t)m, s = 0;
+    double v = c;
+    if (e < cnt) {
+      if (k == kD) {
+        const int r = lo + e;
+        s = 2 * P + r - 1;
+        v = 2.0 * (r == a ? (double)(1 - a) * ld_c(B, a) : ld_c(B, r));
+      } else if (which == LB_F) {
+        if (k == kJ) {
+          const int w = b + 1 + e;
+          n = P + edge(a, w);
+          s = P + edge(b, w);
+        } else if (e < n1) {
+          const int w = b + 1 + e;
+          n = edge(a, w);
+          s = P + edge(b, w);
+        } else if (e < n2) {
+          const int w = a + 1 + (e - n1);
+          n = edge(w, b);
+          s = P + edge(a, w);
+        } else if (e < n2 + up) {
+          const int w = b + 1 + (e - n2);
+          n = edge(b, w);
+          s = P + edge(a, w);
+        } else {
+          const int l = lo + (e - n2 - up);
+          n = P + eab;
+          s = 2 * P + l - 1;
+          v = delta(B, a, l) - delta(B, b, l);
+        }
+      } else {
+        if (e < n1) {
+          const int l = lo + e;
+          s = 2 * P + l - 1;
+          v = delta(B, a, l) + delta(B, b, l);
+        } else if (e < n2) {
+          const int w = b + 1 + (e - n1);
+          n = edge(a, w);
+          s = edge(b, w);
+        } else {
+          const int i = e - n2, w = i < a ? i : i < b - 1 ? i + 1 : i + 2;
+          n = P + edge(a, w);
+          s = P + edge(b, w);
+          if (a < w && w < b) v = -c;
+        }
+      }
+      val[off + e] = v;
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const int word = 32 * t + lane, src = word / 3, q = word - 3 * src;
+      const int32_t nn = __shfl_sync(0xffffffffu, n, src), ss = __shfl_sync(0xffffffffu, s, src);
+      if (e0 + src < cnt) idx[3 * (off + e0) + word] = q == 0 ? (int32_t)m : q == 1 ? nn : ss;
+    }
+  }
 }
 
 // Eq. (02): coef_j = Tr(F_j A) = sum_pq (F_j)_pq A_qp.
@@ -252,15 +279,12 @@ cudaError_t build_tables(int N, int32_t* pair_ab, double* tab, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-cudaError_t structure_count(const lb::BasisView& B, int which, int64_t* per_m, cudaStream_t st) {
-  k_rows<false><<<nblocks(B.M * 32, 256), 256, 0, st>>>(B, which, per_m, nullptr, nullptr, nullptr);
-  note_launch(1);
-  return cudaGetLastError();
+int64_t structure_total(int N, int which) {
+  return rows_s(N, which, N - 1, N) + rows_j(N, which, N - 1, N) + rows_d(N, which, N);
 }
 
-cudaError_t structure_fill(const lb::BasisView& B, int which, const int64_t* offsets,
-                           int32_t* idx3, double* val, cudaStream_t st) {
-  k_rows<true><<<nblocks(B.M * 32, 256), 256, 0, st>>>(B, which, nullptr, offsets, idx3, val);
+cudaError_t structure_fill(const lb::BasisView& B, int which, int32_t* idx3, double* val, cudaStream_t st) {
+  k_rows<<<nblocks(B.M * 32, 256), 256, 0, st>>>(B, which, idx3, val);
   note_launch(1);
   return cudaGetLastError();
 }

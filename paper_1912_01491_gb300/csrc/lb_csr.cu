@@ -896,10 +896,6 @@ static cudaError_t scan_counts(const unsigned long long* cnt, int64_t* off, int6
   return cudaStreamSynchronize(st);
 }
 
-cudaError_t exclusive_scan(const int64_t* counts, int64_t* off, int64_t n, cudaStream_t st) {
-  return scan_device(counts, off, n, st);
-}
-
 // Buckets of terms: counts (M + 1), offsets (M + 1), the terms.
 struct Buckets {
   Buf cnt, off, terms;

@@ -40,9 +40,8 @@ int cuda_fail(cudaError_t e, const char* what);
 
 // kernel (a) and friends (lb_basis.cu)
 cudaError_t build_tables(int N, int32_t* pair_ab, double* tab, cudaStream_t st);
-cudaError_t structure_count(const lb::BasisView& B, int which, int64_t* per_m, cudaStream_t st);
-cudaError_t structure_fill(const lb::BasisView& B, int which, const int64_t* offsets,
-                           int32_t* idx3, double* val, cudaStream_t st);
+int64_t structure_total(int N, int which);
+cudaError_t structure_fill(const lb::BasisView& B, int which, int32_t* idx3, double* val, cudaStream_t st);
 cudaError_t expand(const lb::BasisView& B, const double2* A, double2* coef, cudaStream_t st);
 cudaError_t rho(const lb::BasisView& B, const double* v, double2* out, cudaStream_t st);
 // sum_i v_i F_i (rho without the 1/N identity part)
@@ -80,9 +79,6 @@ int hermitian_eig(const double2* H, int N, double* E, double2* Ub, cudaStream_t 
 // Eigenvalue density on an nre x nim grid over box = {re_lo, re_hi, im_lo, im_hi}.
 cudaError_t spectrum_density(const double2* w, int64_t n, const double* box, int nre, int nim, double* dens,
                              cudaStream_t st);
-// off[0..n] = exclusive prefix sums of n int64 counts (off[n] = total);
-// synchronous with respect to st.
-cudaError_t exclusive_scan(const int64_t* counts, int64_t* off, int64_t n, cudaStream_t st);
 cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP, const double* gamma_host,
                                  const int64_t* lp_ptr_host, const int64_t* lp_idx, const double2* lp_val,
                                  CsrOut* out, cudaStream_t st);
