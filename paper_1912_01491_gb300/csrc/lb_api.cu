@@ -110,6 +110,7 @@ struct lb_system {
   float* scale = nullptr;
   lbi::CsrOut csr;               // LB_CSR: rowptr, col, val, K (K aliases csr.K)
   float* csr32 = nullptr;        // FP32 copy of csr.val, made on first use
+  lbi::CsrPlan plan;             // layout of a CSR system, made on first use
   double ms[LB_PHASES] = {};     // phase times of the call that built it
 };
 
@@ -396,8 +397,25 @@ int lb_rho_checks(const lb_basis_t* b, const double* V, int64_t nsnap, double ps
 
 struct lb_csr {
   lbi::CsrOut m;
+  // what the integrations keep, made under mu (a handle may be used from several threads)
+  std::mutex mu;
   float* val32 = nullptr;
+  lbi::CsrPlan plan;
 };
+
+namespace {
+
+// The layout of a sparse system for one precision; *usable as csr_plan.  FP32
+// systems of longer rows keep the row sums by several lanes: the layout adds in
+// CSR order, which in FP32 would be another rounding.
+cudaError_t csr_view(const lbi::CsrOut& m, lbi::CsrPlan* plan, int precision, cudaStream_t st, lbi::CsrRegView* view,
+                     bool* usable) {
+  *usable = false;
+  if (precision == LB_FP32 && lbi::csr_group_width(m.nnz, m.M) != 1) return cudaSuccess;
+  return lbi::csr_plan(plan, m.M, m.nnz, m.rowptr, m.col, m.val, precision, st, view, usable);
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -472,6 +490,7 @@ int lb_csr_destroy(lb_csr_t* c) {
   cudaFree(c->m.val);
   cudaFree(c->m.K);
   cudaFree(c->val32);
+  lbi::csr_plan_free(&c->plan);
   delete c;
   return LB_OK;
 }
@@ -483,18 +502,25 @@ int lb_rk4_csr(const lb_csr_t* c, int precision, int correct_every, double* v, d
   LB_REQUIRE(nsteps >= 0 && std::isfinite(dt) && correct_every >= 0, "lb_rk4_csr: bad arguments");
   lb_csr* cc = const_cast<lb_csr*>(c);
   const void* val = c->m.val;
-  if (precision == LB_FP32) {
-    if (!cc->val32) {
-      DevBuf b32;
-      int rc;
-      if ((rc = alloc_or_enomem(b32, sizeof(float) * (size_t)(c->m.nnz + 1), "FP32 values")) != LB_OK) return rc;
-      LB_TRY_CUDA(lbi::to_f32(c->m.nnz, c->m.val, b32.as<float>(), S(stream)), "pack FP32 values");
-      cc->val32 = static_cast<float*>(b32.release());
+  lbi::CsrRegView view;
+  bool reg = false;
+  {
+    std::lock_guard<std::mutex> lock(cc->mu);
+    LB_TRY_CUDA(csr_view(c->m, &cc->plan, precision, S(stream), &view, &reg), "lb_rk4_csr: layout");
+    if (!reg && precision == LB_FP32) {
+      if (!cc->val32) {
+        DevBuf b32;
+        int rc;
+        if ((rc = alloc_or_enomem(b32, sizeof(float) * (size_t)(c->m.nnz + 1), "FP32 values")) != LB_OK) return rc;
+        LB_TRY_CUDA(lbi::to_f32(c->m.nnz, c->m.val, b32.as<float>(), S(stream)), "pack FP32 values");
+        LB_TRY_CUDA(cudaStreamSynchronize(S(stream)), "pack FP32 values");  // other streams may use them next
+        cc->val32 = static_cast<float*>(b32.release());
+      }
+      val = cc->val32;
     }
-    val = cc->val32;
   }
   LB_TRY_CUDA(lbi::rk4_csr(c->m.M, precision, c->m.rowptr, c->m.col, val, c->m.val, correct_every, c->m.K, v, dt,
-                           nsteps, work, S(stream)),
+                           nsteps, work, S(stream), reg ? &view : nullptr),
               "lb_rk4_csr");
   return LB_OK;
 }
@@ -516,8 +542,21 @@ int lb_rk4_csr_td(const lb_csr_t* A0, const lb_csr_t* Q1, int nseg, const double
                "lb_rk4_csr_td: seg_start must increase within [0, period)");
   }
   LB_REQUIRE(nsteps >= 0 && dt > 0 && std::isfinite(dt), "lb_rk4_csr_td: bad step count or dt");
+  lbi::CsrRegView v0, v1;
+  bool reg = false, reg1 = false;
+  {
+    lb_csr* c = const_cast<lb_csr*>(A0);
+    std::lock_guard<std::mutex> lock(c->mu);
+    LB_TRY_CUDA(csr_view(A0->m, &c->plan, LB_FP64, S(stream), &v0, &reg), "lb_rk4_csr_td: layout");
+  }
+  if (reg) {
+    lb_csr* c = const_cast<lb_csr*>(Q1);
+    std::lock_guard<std::mutex> lock(c->mu);
+    LB_TRY_CUDA(csr_view(Q1->m, &c->plan, LB_FP64, S(stream), &v1, &reg1), "lb_rk4_csr_td: layout");
+  }
   LB_TRY_CUDA(lbi::rk4_csr_td(A0->m.M, A0->m.rowptr, A0->m.col, A0->m.val, Q1->m.rowptr, Q1->m.col, Q1->m.val,
-                              A0->m.K, nseg, seg_start, seg_eps, period, t0, v, dt, nsteps, work, S(stream)),
+                              A0->m.K, nseg, seg_start, seg_eps, period, t0, v, dt, nsteps, work, S(stream),
+                              reg && reg1 ? &v0 : nullptr, reg && reg1 ? &v1 : nullptr),
               "lb_rk4_csr_td");
   return LB_OK;
 }
@@ -898,6 +937,7 @@ int lb_system_destroy(lb_system_t* s) {
   cudaFree(s->csr.val);
   cudaFree(s->csr.K);
   cudaFree(s->csr32);
+  lbi::csr_plan_free(&s->plan);
   delete s;
   return LB_OK;
 }
@@ -1151,7 +1191,13 @@ static int integrate_steps(lb_system_t* s, int precision, int correct_every, con
                precision);
   }
   const void* Ap = s->format == LB_CSR ? (const void*)s->csr.val : (const void*)s->A;
-  if (precision == LB_FP32 && s->format == LB_CSR) {
+  lbi::CsrRegView view;
+  bool reg = false;
+  if (s->format == LB_CSR)
+    LB_TRY_CUDA(csr_view(s->csr, &s->plan, precision, c.st, &view, &reg), "lb_integrate: layout");
+  if (reg) {
+    // the layout holds the values
+  } else if (precision == LB_FP32 && s->format == LB_CSR) {
     if (!s->csr32) {
       DevBuf b32;
       if ((rc = alloc_or_enomem(b32, sizeof(float) * (size_t)(s->csr.nnz + 1), "FP32 values")) != LB_OK) return rc;
@@ -1189,7 +1235,7 @@ static int integrate_steps(lb_system_t* s, int precision, int correct_every, con
     const int64_t nseg = nsnap > 0 ? nsnap : 1;
     for (int64_t i = 0; i < nseg; ++i) {
       LB_TRY_CUDA(lbi::rk4_csr(M, precision, s->csr.rowptr, s->csr.col, Ap, s->csr.val, correct_every, s->csr.K,
-                               dv.as<double>(), dt, seg, work.p, c.st),
+                               dv.as<double>(), dt, seg, work.p, c.st, reg ? &view : nullptr),
                   "RK4 (CSR)");
       if (nsnap > 0)
         LB_TRY_CUDA(cudaMemcpyAsync(dsn.as<double>() + (size_t)i * M, dv.p, 8 * (size_t)M, cudaMemcpyDeviceToDevice,

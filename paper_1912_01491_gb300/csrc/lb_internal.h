@@ -82,14 +82,53 @@ cudaError_t spectrum_density(const double2* w, int64_t n, const double* box, int
 cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP, const double* gamma_host,
                                  const int64_t* lp_ptr_host, const int64_t* lp_idx, const double2* lp_val,
                                  CsrOut* out, cudaStream_t st);
+cudaError_t to_f32(int64_t n, const double* x, float* y, cudaStream_t st);
+
+// The layout of a sparse system by groups of 32 rows (lb_csr_reg.cu), made at
+// the first integration of a system and kept with it.
+struct CsrPlan {
+  int state = 0;  // 0: not looked at, 1: made, -1: the pattern does not suit it
+  int64_t slots = 0, nlong = 0, nexp = 0;
+  int32_t *rec = nullptr, *delta = nullptr, *ecol = nullptr, *longrow = nullptr, *egroup = nullptr;
+  uint8_t* len8 = nullptr;
+  void *val[2] = {nullptr, nullptr}, *eval[2] = {nullptr, nullptr};  // FP64, FP32
+};
+struct CsrRegView {
+  const int32_t *rec, *delta;
+  const uint8_t* len8;
+  const int32_t *ecol, *longrow, *egroup;
+  int64_t nlong, nexp;  // long rows, explicit groups
+  const void *val, *eval;
+  int64_t nnz;
+  const int64_t* rowptr;  // the CSR arrays
+  const int32_t* col;
+  const double* val64;
+};
+// Makes what precision needs; *usable = false (no error): the pattern does not
+// suit the layout, or there is no memory for it.  Synchronous with respect to
+// st when it makes anything.
+cudaError_t csr_plan(CsrPlan* p, int64_t M, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                     int precision, cudaStream_t st, CsrRegView* view, bool* usable);
+void csr_plan_free(CsrPlan* p);
+// Lanes per CSR row of the kernels without a layout (1: rows summed in order).
+int csr_group_width(int64_t nnz, int64_t M);
+// One stage for A (+ eps Q1, FP64); x and xn FP64 or FP32 as precision; h:
+// dt/2, dt/2, dt, dt/6.
+cudaError_t csr_reg_stage(int precision, int stage, int64_t M, const CsrRegView& A, const CsrRegView* Q1, double eps,
+                          const double* Keff, const void* x, void* xn, double* acc, double* v, double h,
+                          cudaStream_t st);
+cudaError_t csr_reg_correction(int64_t M, const CsrRegView& A, const double* v, const double* K, double* Keff,
+                               cudaStream_t st);
+
+// reg: the system's layout, or null (val: FP64 or FP32 values in CSR order).
 cudaError_t rk4_csr(int64_t M, int precision, const int64_t* rowptr, const int32_t* col, const void* val,
                     const double* val64, int correct_every, const double* K, double* v, double dt, int64_t nsteps,
-                    void* work, cudaStream_t st);
-cudaError_t to_f32(int64_t n, const double* x, float* y, cudaStream_t st);
+                    void* work, cudaStream_t st, const CsrRegView* reg = nullptr);
 cudaError_t rk4_csr_td(int64_t M, const int64_t* rowptr, const int32_t* col, const double* val,
                        const int64_t* rowptr1, const int32_t* col1, const double* val1, const double* K, int nseg,
                        const double* seg_start, const double* seg_eps, double T, double t0, double* v, double dt,
-                       int64_t nsteps, void* work, cudaStream_t st);
+                       int64_t nsteps, void* work, cudaStream_t st, const CsrRegView* reg = nullptr,
+                       const CsrRegView* reg1 = nullptr);
 
 // RK4 (lb_rk4.cu)
 cudaError_t pack_fp32(int64_t M, const double* A, float* A32, cudaStream_t st);

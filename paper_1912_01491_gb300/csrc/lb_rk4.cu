@@ -25,7 +25,24 @@
 #include "lb_internal.h"
 #include "lb_rowsum.cuh"
 
+namespace lbi {
+
+// Lanes per CSR row: the largest power of two W <= 32 with four or more
+// entries per lane on average (W = 1: the block-staged thread-per-row form).
+// Short rows favour one thread per row, which keeps 32 rows' loads in flight
+// per warp instruction; long rows favour lanes that share a row's entries.
+int csr_group_width(int64_t nnz, int64_t M) {
+  const double mean = M > 0 ? (double)nnz / (double)M : 0.0;
+  int w = 1;
+  while (w < 32 && 4.0 * (2 * w) <= mean) w *= 2;
+  return w;
+}
+
+}  // namespace lbi
+
 namespace {
+
+using lbi::csr_group_width;
 
 constexpr int kWarpsPerBlock = 8;
 
@@ -779,17 +796,6 @@ cudaError_t run_steps(int64_t M, const void* Ap, const float* scale, const doubl
   return cudaGetLastError();
 }
 
-// Lanes per CSR row: the largest power of two W <= 32 with four or more
-// entries per lane on average (W = 1: the block-staged thread-per-row form).
-// Short rows favour one thread per row, which keeps 32 rows' loads in flight
-// per warp instruction; long rows favour lanes that share a row's entries.
-int csr_group_width(int64_t nnz, int64_t M) {
-  const double mean = M > 0 ? (double)nnz / (double)M : 0.0;
-  int w = 1;
-  while (w < 32 && 4.0 * (2 * w) <= mean) w *= 2;
-  return w;
-}
-
 // Staging capacity (entries) of k_stage_csr_blk: 1.5 times a block's mean
 // range plus one row of slack, within 48 KB of shared memory.
 int csr_stage_cap(int64_t nnz, int64_t M, size_t entry_bytes) {
@@ -942,8 +948,21 @@ namespace lbi {
 cudaError_t rk4_csr_td(int64_t M, const int64_t* rowptr, const int32_t* col, const double* val,
                        const int64_t* rowptr1, const int32_t* col1, const double* val1, const double* K, int nseg,
                        const double* seg_start, const double* seg_eps, double T, double t0, double* v, double dt,
-                       int64_t nsteps, void* work, cudaStream_t st) {
+                       int64_t nsteps, void* work, cudaStream_t st, const CsrRegView* reg, const CsrRegView* reg1) {
   Work w = carve(work, M);
+  if (reg && reg1) {
+    cudaError_t e = cudaMemcpyAsync(w.X, v, sizeof(double) * M, cudaMemcpyDeviceToDevice, st);
+    for (int64_t n = 0; n < nsteps && e == cudaSuccess; ++n) {
+      const double t = t0 + (double)n * dt;
+      const double e1 = eps_at(t + 1e-6 * dt, nseg, seg_start, seg_eps, T);
+      const double e2 = eps_at(t + 0.5 * dt, nseg, seg_start, seg_eps, T);
+      const double e4 = eps_at(t + dt - 1e-6 * dt, nseg, seg_start, seg_eps, T);
+      for (int q = 1; q <= 4 && e == cudaSuccess; ++q)
+        e = csr_reg_stage(LB_FP64, q, M, *reg, reg1, q == 1 ? e1 : q == 4 ? e4 : e2, K, q & 1 ? w.X : w.Y,
+                          q & 1 ? w.Y : w.X, w.acc, v, q < 3 ? 0.5 * dt : q == 3 ? dt : dt / 6.0, st);
+    }
+    return e;
+  }
   const unsigned grid = (unsigned)((M + 255) / 256);
   int64_t nnz = 0;
   cudaError_t e = cudaMemcpyAsync(&nnz, rowptr + M, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
@@ -991,8 +1010,26 @@ cudaError_t rk4_csr_td(int64_t M, const int64_t* rowptr, const int32_t* col, con
 
 cudaError_t rk4_csr(int64_t M, int precision, const int64_t* rowptr, const int32_t* col, const void* val,
                     const double* val64, int correct_every, const double* K, double* v, double dt, int64_t nsteps,
-                    void* work, cudaStream_t st) {
+                    void* work, cudaStream_t st, const CsrRegView* reg) {
   Work w = carve(work, M);
+  if (reg) {
+    const bool f64 = precision == LB_FP64, correct = !f64 && correct_every > 0;
+    cudaError_t e = cudaMemcpyAsync(w.Keff, K, sizeof(double) * M, cudaMemcpyDeviceToDevice, st);
+    void* X = f64 ? static_cast<void*>(w.X) : w.X32;
+    void* Y = f64 ? static_cast<void*>(w.Y) : w.Y32;
+    if (e == cudaSuccess)
+      e = f64 ? cudaMemcpyAsync(X, v, sizeof(double) * M, cudaMemcpyDeviceToDevice, st) : to_f32(M, v, w.X32, st);
+    for (int64_t t = 0; t < nsteps && e == cudaSuccess; ++t) {
+      if (correct && t % correct_every == 0) e = csr_reg_correction(M, *reg, v, K, w.Keff, st);
+      for (int q = 1; q <= 4 && e == cudaSuccess; ++q)
+        e = csr_reg_stage(precision, q, M, *reg, nullptr, 0.0, w.Keff, q & 1 ? X : Y, q & 1 ? Y : X, w.acc, v,
+                          q < 3 ? 0.5 * dt : q == 3 ? dt : dt / 6.0, st);
+    }
+    // short rows and an aligned v: finished when the call returns, as without the layout
+    if (e == cudaSuccess && csr_group_width(reg->nnz, M) == 1 && (reinterpret_cast<uintptr_t>(v) & 15u) == 0)
+      e = cudaStreamSynchronize(st);
+    return e;
+  }
   if (precision == LB_FP64)
     return run_steps_csr<LB_FP64>(M, rowptr, col, val, val64, correct_every, K, v, dt, nsteps, w, st);
   if (precision == LB_FP32)
