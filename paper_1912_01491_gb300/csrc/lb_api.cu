@@ -485,10 +485,7 @@ int lb_csr_copy(const lb_csr_t* c, int64_t* rowptr, int32_t* col, double* val, d
 
 int lb_csr_destroy(lb_csr_t* c) {
   if (!c) return LB_OK;
-  cudaFree(c->m.rowptr);
-  cudaFree(c->m.col);
-  cudaFree(c->m.val);
-  cudaFree(c->m.K);
+  lbi::csr_out_free(&c->m);
   cudaFree(c->val32);
   lbi::csr_plan_free(&c->plan);
   delete c;
@@ -710,6 +707,9 @@ int lb_host_release(void) {
   LB_TRY_CUDA(host_ctx(&c), "lb_host_release");
   LB_TRY_CUDA(cudaStreamSynchronize(c.st), "lb_host_release");
   LB_TRY_CUDA(cudaMemPoolTrimTo(c.pool, 0), "lb_host_release");
+  cudaMemPool_t scratch = nullptr;
+  LB_TRY_CUDA(lbi::scratch_pool(&scratch), "lb_host_release");
+  LB_TRY_CUDA(cudaMemPoolTrimTo(scratch, 0), "lb_host_release");
   return LB_OK;
 }
 
@@ -932,10 +932,7 @@ int lb_system_destroy(lb_system_t* s) {
     pool_free(s->Abf, c.st);
     pool_free(s->scale, c.st);
   }
-  cudaFree(s->csr.rowptr);
-  cudaFree(s->csr.col);
-  cudaFree(s->csr.val);
-  cudaFree(s->csr.K);
+  lbi::csr_out_free(&s->csr);
   cudaFree(s->csr32);
   lbi::csr_plan_free(&s->plan);
   delete s;

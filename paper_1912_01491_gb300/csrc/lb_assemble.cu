@@ -2578,8 +2578,13 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
   // diagonal rows and the diagonal x diagonal tables
   double* scratch = nullptr;
   const size_t dd_at = 3 * (size_t)N * N + N;
-  if (closed && e == cudaSuccess && (dense_out || K))
-    e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), sizeof(double) * (dd_at + DDTables::doubles(N)), st);
+  if (closed && e == cudaSuccess && (dense_out || K)) {
+    // from the retained pool: after a synchronization the default one would go to the driver again (0.15 ms)
+    cudaMemPool_t pool = nullptr;
+    if ((e = scratch_pool(&pool)) == cudaSuccess)
+      e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch),
+                                  sizeof(double) * (dd_at + DDTables::doubles(N)), pool, st);
+  }
   // 3: diagonal x diagonal (closed: cells of constant coefficient from row,
   //    column and corner sums)
   if (dense_out && e == cudaSuccess && N >= 2) {

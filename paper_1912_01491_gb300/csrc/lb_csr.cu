@@ -24,6 +24,10 @@
 //      writes the columns in ascending order with their values.
 // Duplicate terms (the same (l, n) from several j) are summed in the order
 // the fill placed them, so values are reproducible to rounding only.
+#include <algorithm>
+#include <mutex>
+#include <vector>
+
 #include "lb_internal.h"
 
 namespace {
@@ -122,11 +126,16 @@ struct BTerm {
 
 // Count mode (out == nullptr): one more term in bucket b.  Fill mode: the
 // term goes to off[b] + (the bucket's cursor, advanced atomically).
+// keep (may be null): only buckets b with keep[b]; mark: x of every term taken.
 struct Bucketer {
   unsigned long long* cnt;  // count, then cursor (reset to 0 between the passes)
   const int64_t* off;
   BTerm* out;
+  const uint8_t* keep;
+  uint8_t* mark;
   __device__ __forceinline__ void put(int64_t b, int p, int64_t x, double re, double im, double mag) const {
+    if (keep && !keep[b]) return;
+    if (mark) mark[x] = 1;
     const unsigned long long k = atomicAdd(cnt + b, 1ull);
     if (out) out[off[b] + (int64_t)k] = BTerm{p, (int32_t)x, re, im, mag};
   }
@@ -485,8 +494,10 @@ constexpr int kLongCap = 8192;        // hash slots of one block (long rows), pe
 constexpr int kLongThreads = 256;
 constexpr int32_t kEmpty = -1;
 
+// The rows at hand: s = list[i], i < rows (list null: all rows).
 struct RowInputs {
-  int64_t M;
+  int64_t rows;
+  const int64_t* list;
   const double* gamma;
   const int64_t *woff, *uoff, *qoff;  // bucket offsets (M + 1 each; qoff may be null)
   const BTerm *w, *u, *q;
@@ -731,8 +742,9 @@ __device__ __forceinline__ int warp_compact(int32_t* keys, double* val, double* 
 __global__ void __launch_bounds__(kRowWarps * 32) k_row_terms(RowInputs I, unsigned long long* bound,
                                                              int64_t* longlist, unsigned long long* nlong) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t s = (int64_t)blockIdx.x * kRowWarps + wid;
-  if (s >= I.M) return;
+  const int64_t i = (int64_t)blockIdx.x * kRowWarps + wid;
+  if (i >= I.rows) return;
+  const int64_t s = I.list ? I.list[i] : i;
   int64_t t = row_terms(I, s, lane, 32);
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) {
@@ -752,8 +764,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_warp(RowInputs I, const
   __shared__ double val_s[kRowWarps][kRowCap], mag_s[kRowWarps][kRowCap];
   __shared__ WStage ws_s[kRowWarps][32];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t s = (int64_t)blockIdx.x * kRowWarps + wid;
-  if (s >= I.M) return;
+  const int64_t i = (int64_t)blockIdx.x * kRowWarps + wid;
+  if (i >= I.rows) return;
+  const int64_t s = I.list ? I.list[i] : i;
   const unsigned long long tb = bound[s];
   if (tb > (unsigned long long)kRowBound) return;
   int cap = 64;
@@ -829,19 +842,20 @@ __global__ void __launch_bounds__(kLongThreads) k_rows_long(RowInputs I, const i
 // Rows from the scratch ranges to their CSR place in ascending column order
 // (one warp per row; an entry's rank is the number of the row's entries with
 // a smaller column).
-__global__ void __launch_bounds__(256) k_rows_copy(int64_t M, const int64_t* tmpoff, const int32_t* tcol,
+__global__ void __launch_bounds__(256) k_rows_copy(int64_t rows, const int64_t* list, const int64_t* tmpoff, const int32_t* tcol,
                                                   const double* tval, const int64_t* rowptr, int32_t* col,
                                                   double* val) {
-  const int64_t s = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (s >= M) return;
+  if (i >= rows) return;
+  const int64_t s = list ? list[i] : i;
   const int64_t src = tmpoff[s], dst = rowptr[s], k = rowptr[s + 1] - rowptr[s];
-  for (int64_t i = lane; i < k; i += 32) {
-    const int32_t ki = tcol[src + i];
+  for (int64_t q = lane; q < k; q += 32) {
+    const int32_t kq = tcol[src + q];
     int64_t rank = 0;
-    for (int64_t j = 0; j < k; ++j) rank += tcol[src + j] < ki ? 1 : 0;
-    col[dst + rank] = ki;
-    val[dst + rank] = tval[src + i];
+    for (int64_t j = 0; j < k; ++j) rank += tcol[src + j] < kq ? 1 : 0;
+    col[dst + rank] = kq;
+    val[dst + rank] = tval[src + q];
   }
 }
 
@@ -851,13 +865,72 @@ inline unsigned nb(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 namespace lbi {
 
-// Owning device allocation helper for this file (freed on scope exit).
+// The scratch pool of a device: temporaries of the assemblies, and the arrays
+// of sparse systems.  It keeps up to kScratchKeep between calls (a cudaMalloc or
+// cudaFree of the sizes here takes 0.1 to several ms and synchronizes the
+// device; the ladder at N = 2000 spent 10 of its 41 ms in them), the rest goes
+// back at the next synchronization, all of it with lb_host_release.
+constexpr uint64_t kScratchKeep = uint64_t(1) << 30;
+
+cudaError_t scratch_pool(cudaMemPool_t* out) {
+  static std::mutex mu;
+  static std::vector<cudaMemPool_t> pools;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  if ((int)pools.size() <= dev) pools.resize(dev + 1, nullptr);
+  if (!pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+    uint64_t keep = kScratchKeep;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    pools[dev] = p;
+  }
+  *out = pools[dev];
+  return cudaSuccess;
+}
+
+void csr_out_free(CsrOut* m) {
+  if (!m->rowptr) return;
+  cudaDeviceSynchronize();  // kernels of any stream may still read the arrays
+  cudaFree(m->rowptr);
+  cudaFree(m->col);
+  cudaFree(m->val);
+  cudaFree(m->K);
+  *m = CsrOut{};
+}
+
+// Owning device allocation of this file, stream-ordered on st.
+// Sizes the pool would hand back at every synchronization come from cudaMalloc
+// (faster there: 41 against 54 ms for the 7 GB of the ladder at N = 2000).
 struct Buf {
   void* p = nullptr;
+  cudaStream_t st;
+  bool large = false;
+  explicit Buf(cudaStream_t s) : st(s) {}
+  Buf(const Buf&) = delete;
+  Buf& operator=(const Buf&) = delete;
   ~Buf() {
-    if (p) cudaFree(p);
+    if (p && large) cudaFree(p);
+    else if (p) cudaFreeAsync(p, st);
   }
-  cudaError_t alloc(size_t n) { return cudaMalloc(&p, n ? n : 16); }
+  cudaError_t alloc(size_t n) {
+    if (n > kScratchKeep / 2) {
+      large = true;
+      return cudaMalloc(&p, n);
+    }
+    cudaMemPool_t pool = nullptr;
+    const cudaError_t e = scratch_pool(&pool);
+    return e == cudaSuccess ? cudaMallocFromPoolAsync(&p, n ? n : 16, pool, st) : e;
+  }
   template <class T>
   T* as() const {
     return static_cast<T*>(p);
@@ -874,7 +947,7 @@ struct Buf {
 template <class C>
 static cudaError_t scan_device(const C* cnt, int64_t* off, int64_t n, cudaStream_t st) {
   const int64_t nt = (n + kScanTile - 1) / kScanTile;
-  Buf ts;
+  Buf ts(st);
   CK(ts.alloc(sizeof(int64_t) * (size_t)(nt + 1)));
   if (nt > 0) {
     k_scan_tiles<C><<<(unsigned)nt, kScanThreads, 0, st>>>(cnt, n, off, ts.as<int64_t>(), 0);
@@ -884,8 +957,7 @@ static cudaError_t scan_device(const C* cnt, int64_t* off, int64_t n, cudaStream
   } else {
     CK(cudaMemsetAsync(off, 0, sizeof(int64_t), st));
   }
-  // the tile sums are freed when this returns: the scan must be complete
-  return cudaStreamSynchronize(st);
+  return cudaGetLastError();
 }
 
 // The same, and *total (host) = off[n].
@@ -900,19 +972,21 @@ static cudaError_t scan_counts(const unsigned long long* cnt, int64_t* off, int6
 struct Buckets {
   Buf cnt, off, terms;
   int64_t total = 0;
+  explicit Buckets(cudaStream_t st) : cnt(st), off(st), terms(st) {}
 };
 
 // Count with `emit(bucketer)`, scan, reset the cursors, fill with `emit`.
 template <class Emit>
-static cudaError_t build_buckets(int64_t M, Buckets& b, Emit emit, cudaStream_t st) {
+static cudaError_t build_buckets(int64_t M, Buckets& b, const uint8_t* keep, uint8_t* mark, Emit emit,
+                                 cudaStream_t st) {
   CK(b.cnt.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
   CK(b.off.alloc(sizeof(int64_t) * (size_t)(M + 1)));
   CK(cudaMemsetAsync(b.cnt.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
-  CK(emit(Bucketer{b.cnt.as<unsigned long long>(), nullptr, nullptr}));
+  CK(emit(Bucketer{b.cnt.as<unsigned long long>(), nullptr, nullptr, keep, mark}));
   CK(scan_counts(b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), M, &b.total, st));
   CK(b.terms.alloc(sizeof(BTerm) * (size_t)b.total));
   CK(cudaMemsetAsync(b.cnt.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
-  if (b.total > 0) CK(emit(Bucketer{b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), b.terms.as<BTerm>()}));
+  if (b.total > 0) CK(emit(Bucketer{b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), b.terms.as<BTerm>(), keep, nullptr}));
   return cudaSuccess;
 }
 
@@ -921,7 +995,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
                                  CsrOut* out, cudaStream_t st) {
   const int64_t M = B.M;
   const int64_t nu = lp_ptr_host[nP];
-  Buf dptr, dgamma;
+  Buf dptr(st), dgamma(st);
   CK(dptr.alloc(sizeof(int64_t) * (nP + 1)));
   CK(dgamma.alloc(sizeof(double) * (nP > 0 ? nP : 1)));
   CK(cudaMemcpyAsync(dptr.p, lp_ptr_host, sizeof(int64_t) * (nP + 1), cudaMemcpyHostToDevice, st));
@@ -929,7 +1003,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   const int64_t* dp = dptr.as<int64_t>();
   // ---- diagonal components of the channels: dense per channel, suffix sums
   const int N = B.N;
-  Buf dl, hasD, suf, sufm;
+  Buf dl(st), hasD(st), suf(st), sufm(st);
   CK(dl.alloc(sizeof(double2) * (size_t)nP * N));
   CK(hasD.alloc(sizeof(int) * (size_t)(nP > 0 ? nP : 1)));
   CK(suf.alloc(sizeof(double2) * (size_t)nP * N));
@@ -944,9 +1018,33 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   }
   const int64_t ndp = (int64_t)nP * N, ndd = (int64_t)nP * (N - 1) * (N - 1);
   const int S = fiber_slices(N);
+  // ---- rows in closed form: their counts, and the list of the rows that are left.  Below 64 levels too many rows
+  // are near the diagonal for the extra launches to pay; more channels than four have no tables
+  const bool bulk = N >= 64 && nP <= 4 && csr_bulk_bytes(N, nP) <= kScratchKeep / 2;
+  Buf bmem(st), rowc(st), list(st), need(st), bctr(st);  // bctr: [0] join terms, [1] rows left
+  CsrBulk cb{};
+  CK(rowc.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
+  unsigned long long hb[2] = {0, (unsigned long long)M};
+  if (bulk) {
+    CK(bmem.alloc(csr_bulk_bytes(N, nP)));
+    CK(list.alloc(sizeof(int64_t) * (size_t)M));
+    CK(need.alloc((size_t)M));
+    CK(bctr.alloc(sizeof(hb)));
+    CK(cudaMemsetAsync(bctr.p, 0, sizeof(hb), st));
+    CK(cudaMemsetAsync(need.p, 0, (size_t)M, st));
+    CK(cudaMemsetAsync(rowc.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
+    cb = csr_bulk_carve(bmem.p, N, nP, dgamma.as<double>());
+    unsigned long long* bc = bctr.as<unsigned long long>();
+    CK(csr_bulk_count(B, cb, nP, dp, lp_idx, lp_val, nu, dl.as<double2>(), hasD.as<int>(), h,
+                      rowc.as<unsigned long long>(), bc, list.as<int64_t>(), bc + 1, st));
+    CK(cudaMemcpyAsync(hb, bctr.p, sizeof(hb), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+  }
+  const uint8_t* slow = bulk ? cb.slow : nullptr;
+  const int64_t rows = (int64_t)hb[1];
   // ---- W (by column s), U (by row l), Q (by row s)
-  Buckets W, U, Q;
-  CK(build_buckets(M, W, [&](Bucketer bk) {
+  Buckets W(st), U(st), Q(st);
+  CK(build_buckets(M, W, slow, bulk ? need.as<uint8_t>() : nullptr, [&](Bucketer bk) {
     if (nu > 0) {
       k_w_bucket<<<nb(nu * S, 256), 256, 0, st>>>(B, nP, dp, lp_idx, lp_val, nu, bk);
       k_dpart_bucket<<<nb(ndp, 128), 128, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
@@ -955,7 +1053,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
     }
     return cudaGetLastError();
   }, st));
-  CK(build_buckets(M, U, [&](Bucketer bk) {
+  CK(build_buckets(M, U, bulk ? need.as<uint8_t>() : nullptr, nullptr, [&](Bucketer bk) {
     if (nu > 0) {
       k_u_bucket<<<nb(nu * S, 256), 256, 0, st>>>(B, nP, dp, lp_idx, lp_val, nu, bk);
       k_dpart_bucket<<<nb(ndp, 128), 128, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
@@ -970,7 +1068,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
     return cudaGetLastError();
   }, st));
   if (h) {
-    Buf hlist, hcount;
+    Buf hlist(st), hcount(st);
     CK(hlist.alloc(sizeof(int64_t) * (size_t)(2 * B.P)));
     CK(hcount.alloc(sizeof(unsigned long long)));
     CK(cudaMemsetAsync(hcount.p, 0, sizeof(unsigned long long), st));
@@ -979,7 +1077,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
     unsigned long long nh = 0;
     CK(cudaMemcpyAsync(&nh, hcount.p, sizeof(nh), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    CK(build_buckets(M, Q, [&](Bucketer bk) {
+    CK(build_buckets(M, Q, slow, nullptr, [&](Bucketer bk) {
       if (nh > 0) {
         k_q_pair_bucket<<<nb((int64_t)nh * S, 256), 256, 0, st>>>(B, h, hlist.as<int64_t>(), (int64_t)nh, bk);
         note_launch(1);
@@ -990,17 +1088,18 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
     }, st));
   }
   // ---- rows: term bounds, one accumulation into scratch ranges, CSR
-  RowInputs I{M, dgamma.as<double>(), W.off.as<int64_t>(), U.off.as<int64_t>(), h ? Q.off.as<int64_t>() : nullptr,
+  RowInputs I{rows, bulk ? list.as<int64_t>() : nullptr, dgamma.as<double>(), W.off.as<int64_t>(), U.off.as<int64_t>(), h ? Q.off.as<int64_t>() : nullptr,
               W.terms.as<BTerm>(), U.terms.as<BTerm>(), h ? Q.terms.as<BTerm>() : nullptr};
-  Buf bound, tmpoff, longlist, ctr;  // ctr: [0] long rows, [1] status
+  Buf bound(st), tmpoff(st), longlist(st), ctr(st);  // ctr: [0] long rows, [1] status
   CK(bound.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
   CK(tmpoff.alloc(sizeof(int64_t) * (size_t)(M + 1)));
   CK(longlist.alloc(sizeof(int64_t) * (size_t)M));
   CK(ctr.alloc(sizeof(unsigned long long) * 2));
   CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned long long) * 2, st));
+  if (bulk) CK(cudaMemsetAsync(bound.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
   unsigned long long* c = ctr.as<unsigned long long>();
   int* status = reinterpret_cast<int*>(c + 1);
-  const unsigned rgrid = nb(M, kRowWarps);
+  const unsigned rgrid = std::max(nb(rows, kRowWarps), 1u);
   k_row_terms<<<rgrid, kRowWarps * 32, 0, st>>>(I, bound.as<unsigned long long>(), longlist.as<int64_t>(), c);
   note_launch(1);
   int64_t nterms = 0;
@@ -1009,10 +1108,9 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   CK(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   const int64_t nlong = (int64_t)hc[0];
-  Buf tcol, tval, rowc;
+  Buf tcol(st), tval(st);
   CK(tcol.alloc(sizeof(int32_t) * (size_t)(nterms + 1)));
   CK(tval.alloc(sizeof(double) * (size_t)(nterms + 1)));
-  CK(rowc.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
   k_rows_warp<<<rgrid, kRowWarps * 32, 0, st>>>(I, bound.as<unsigned long long>(), tmpoff.as<int64_t>(),
                                                 tcol.as<int32_t>(), tval.as<double>(), rowc.as<unsigned long long>(),
                                                 status);
@@ -1026,20 +1124,21 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
                                                              rowc.as<unsigned long long>(), status);
     note_launch(1);
   }
-  Buf rowptr;
+  Buf rowptr(st);
   CK(rowptr.alloc(sizeof(int64_t) * (size_t)(M + 1)));
   int64_t nnz = 0;
   CK(scan_counts(rowc.as<unsigned long long>(), rowptr.as<int64_t>(), M, &nnz, st));
   CK(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (hc[1] != 0) return cudaErrorNotSupported;  // a row has more than kLongCap distinct columns
-  Buf col, val, K;
+  Buf col(st), val(st), K(st);
   CK(col.alloc(sizeof(int32_t) * (size_t)(nnz + 1)));
   CK(val.alloc(sizeof(double) * (size_t)(nnz + 1)));
   CK(K.alloc(sizeof(double) * (size_t)M));
-  k_rows_copy<<<nb(M, 8), 256, 0, st>>>(M, tmpoff.as<int64_t>(), tcol.as<int32_t>(), tval.as<double>(),
+  k_rows_copy<<<std::max(nb(rows, 8), 1u), 256, 0, st>>>(rows, I.list, tmpoff.as<int64_t>(), tcol.as<int32_t>(), tval.as<double>(),
                                         rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>());
   note_launch(1);
+  if (bulk) CK(csr_bulk_fill(B, cb, nP, rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>(), st));
   // ---- K
   CK(cudaMemsetAsync(K.p, 0, sizeof(double) * M, st));
   int64_t maxn = 0;
@@ -1061,7 +1160,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   val.p = nullptr;
   out->K = K.as<double>();
   K.p = nullptr;
-  out->terms = nterms;
+  out->terms = nterms + (int64_t)hb[0];
   return cudaSuccess;
 }
 

@@ -79,6 +79,36 @@ int hermitian_eig(const double2* H, int N, double* E, double2* Ub, cudaStream_t 
 // Eigenvalue density on an nre x nim grid over box = {re_lo, re_hi, im_lo, im_hi}.
 cudaError_t spectrum_density(const double2* w, int64_t n, const double* box, int nre, int nim, double* dens,
                              cudaStream_t st);
+// Rows of a sparse system in closed form (lb_csr_bulk.cu): tables on the graphs
+// of the l_p and of H, in one allocation of csr_bulk_bytes.
+struct CsrBulk {
+  double2* L;           // nP x N x N
+  double* mag;          // nP x N x N: sum of |l| on the edge
+  int* cnt;             // N x N: list entries on the edge
+  uint8_t* near;        // N x N: 1: the rows of this pair go the general way
+  double *smax, *mx, *gd;
+  int* maxdeg;
+  double* hdiag;        // N
+  int* ucol;            // candidates of a vertex, and G, L_p at them
+  double2 *G, *Lu;
+  int *nbr, *nbc;       // neighbours on the l graph and their list entries
+  int *deg, *nn1, *nh, *d1, *npd;
+  uint8_t* slow;        // M: 1: the row goes the general way
+  const double* gamma;  // nP, device
+  size_t zeroed;
+};
+size_t csr_bulk_bytes(int N, int nP);
+CsrBulk csr_bulk_carve(void* mem, int N, int nP, const double* gamma);
+cudaError_t csr_bulk_count(const lb::BasisView& B, const CsrBulk& b, int nP, const int64_t* lp_ptr,
+                           const int64_t* lp_idx, const double2* lp_val, int64_t nu, const double2* dl, const int* hasD,
+                           const double* h, unsigned long long* rowc, unsigned long long* terms, int64_t* list,
+                           unsigned long long* nlist, cudaStream_t st);
+cudaError_t csr_bulk_fill(const lb::BasisView& B, const CsrBulk& b, int nP, const int64_t* rowptr, int32_t* col,
+                          double* val, cudaStream_t st);
+// The device's scratch pool (stream-ordered temporaries and the CsrOut arrays).
+cudaError_t scratch_pool(cudaMemPool_t* out);
+// Frees the arrays; waits for the device first.
+void csr_out_free(CsrOut* m);
 cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP, const double* gamma_host,
                                  const int64_t* lp_ptr_host, const int64_t* lp_idx, const double2* lp_val,
                                  CsrOut* out, cudaStream_t st);
