@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "lb_internal.h"
+#include "lb_rowsum.cuh"
 
 namespace {
 
@@ -41,7 +42,9 @@ using namespace lb;
 __host__ __device__ inline int fiber_slices(int N) { return 2 * N - 1; }
 
 // Slice t of the f-fibre of the pair element k: every (l, s) with
-// f_{k l s} != 0, with the value.
+// f_{k l s} != 0, with a function that computes the value: most entries are
+// only counted, or dropped for their bucket, and FP64 work is what these
+// passes would spend their time on.
 template <class Emit>
 __device__ void f_fiber_slice(const BasisView& B, int64_t k, int t, Emit& emit) {
   const int N = B.N;
@@ -54,7 +57,7 @@ __device__ void f_fiber_slice(const BasisView& B, int64_t k, int t, Emit& emit) 
       const int v = vi ? b : a, vp = vi ? a : b;
       for (int tl = kS; tl <= kJ; ++tl) {
         const Elem el = make_pair(tl, v, w), es = make_pair(1 ^ tk ^ tl, vp, w);
-        emit(elem_index(B, tl, v, w), elem_index(B, es.kind, vp, w), f_value(B, ek, el, es));
+        emit(elem_index(B, tl, v, w), elem_index(B, es.kind, vp, w), [&] { return f_value(B, ek, el, es); });
       }
     }
   } else {
@@ -62,19 +65,26 @@ __device__ void f_fiber_slice(const BasisView& B, int64_t k, int t, Emit& emit) 
     if (lam < imax(a, 1) || lam > b) return;
     const Elem ekb = make_pair(1 - tk, a, b);
     const int64_t kb = partner(B, k);
-    emit(kb, d_index(B, lam), f_value(B, ek, ekb, make_d(lam)));
-    emit(d_index(B, lam), kb, f_value(B, ek, make_d(lam), ekb));
+    emit(kb, d_index(B, lam), [&] { return f_value(B, ek, ekb, make_d(lam)); });
+    emit(d_index(B, lam), kb, [&] { return f_value(B, ek, make_d(lam), ekb); });
   }
 }
 
 // Slice t of the z-fibre of the pair element j: every (l, n) with
-// z_{j l n} != 0, with z = f + i d.
+// z_{j l n} != 0, with z = f + i d (one of the two; likewise as a function).
 template <class Emit>
 __device__ void z_fiber_slice(const BasisView& B, int64_t j, int t, Emit& emit) {
   const int N = B.N;
   const Elem ej = decode(B, j);
   const int a = ej.a, b = ej.b, tj = ej.kind;
-  double f, d;
+  // the f or the d part of z
+  auto part = [&](const Elem& el, const Elem& en, bool isf) {
+    return [&B, ej, el, en, isf] {
+      double f, d;
+      fd_value(B, ej, el, en, f, d);
+      return isf ? make_double2(f, 0.0) : make_double2(0.0, d);
+    };
+  };
   if (t < N) {
     const int w = t;
     if (w == a || w == b) return;
@@ -84,10 +94,8 @@ __device__ void z_fiber_slice(const BasisView& B, int64_t j, int t, Emit& emit) 
         const Elem el = make_pair(tl, v, w);
         const int64_t l = elem_index(B, tl, v, w);
         const Elem enf = make_pair(1 ^ tj ^ tl, vp, w), end = make_pair(tj ^ tl, vp, w);
-        fd_value(B, ej, el, enf, f, d);
-        emit(l, elem_index(B, enf.kind, vp, w), f, 0.0);
-        fd_value(B, ej, el, end, f, d);
-        emit(l, elem_index(B, end.kind, vp, w), 0.0, d);
+        emit(l, elem_index(B, enf.kind, vp, w), part(el, enf, true));
+        emit(l, elem_index(B, end.kind, vp, w), part(el, end, false));
       }
     }
   } else {
@@ -96,16 +104,12 @@ __device__ void z_fiber_slice(const BasisView& B, int64_t j, int t, Emit& emit) 
     const Elem ejb = make_pair(1 - tj, a, b), ed = make_d(lam);
     const int64_t jb = partner(B, j);
     if (lam <= b) {  // f-fibres: (partner(j), D) and (D, partner(j))
-      fd_value(B, ej, ejb, ed, f, d);
-      emit(jb, d_index(B, lam), f, 0.0);
-      fd_value(B, ej, ed, ejb, f, d);
-      emit(d_index(B, lam), jb, f, 0.0);
+      emit(jb, d_index(B, lam), part(ejb, ed, true));
+      emit(d_index(B, lam), jb, part(ed, ejb, true));
     }
     if (!(a == 0 && b == 1 && lam == 1)) {  // d-fibres: (j, D) and (D, j)
-      fd_value(B, ej, ej, ed, f, d);
-      emit(j, d_index(B, lam), 0.0, d);
-      fd_value(B, ej, ed, ej, f, d);
-      emit(d_index(B, lam), j, 0.0, d);
+      emit(j, d_index(B, lam), part(ej, ed, false));
+      emit(d_index(B, lam), j, part(ed, ej, false));
     }
   }
 }
@@ -133,11 +137,16 @@ struct Bucketer {
   BTerm* out;
   const uint8_t* keep;
   uint8_t* mark;
-  __device__ __forceinline__ void put(int64_t b, int p, int64_t x, double re, double im, double mag) const {
-    if (keep && !keep[b]) return;
+  __device__ __forceinline__ bool wants(int64_t b) const { return !keep || keep[b]; }
+  template <class Term>  // term() -> BTerm, called in fill mode only
+  __device__ __forceinline__ void put(int64_t b, int64_t x, Term term) const {
+    if (!wants(b)) return;
     if (mark) mark[x] = 1;
     const unsigned long long k = atomicAdd(cnt + b, 1ull);
-    if (out) out[off[b] + (int64_t)k] = BTerm{p, (int32_t)x, re, im, mag};
+    if (out) out[off[b] + (int64_t)k] = term();
+  }
+  __device__ __forceinline__ void put(int64_t b, int p, int64_t x, double re, double im, double mag) const {
+    put(b, x, [&] { return BTerm{p, (int32_t)x, re, im, mag}; });
   }
 };
 
@@ -153,8 +162,12 @@ __global__ void k_w_bucket(BasisView B, int nP, const int64_t* lp_ptr, const int
   if (k >= 2 * B.P) return;  // diagonal components: k_dpart_bucket
   const int p = channel_of(lp_ptr, nP, u);
   const double2 lk = lp_val[u];
-  const double am = sqrt(lk.x * lk.x + lk.y * lk.y);
-  auto emit = [&](int64_t l, int64_t s, double f) { bk.put(s, p, l, lk.x * f, -lk.y * f, am * fabs(f)); };
+  auto emit = [&](int64_t l, int64_t s, auto value) {
+    bk.put(s, l, [&] {
+      const double f = value(), am = sqrt(lk.x * lk.x + lk.y * lk.y);
+      return BTerm{p, (int32_t)l, lk.x * f, -lk.y * f, am * fabs(f)};
+    });
+  };
   f_fiber_slice(B, k, (int)(it % S), emit);
 }
 
@@ -170,9 +183,12 @@ __global__ void k_u_bucket(BasisView B, int nP, const int64_t* lp_ptr, const int
   if (j >= 2 * B.P) return;  // diagonal components: k_dpart_bucket, k_udd_bucket
   const int p = channel_of(lp_ptr, nP, u);
   const double2 lj = lp_val[u];
-  const double am = sqrt(lj.x * lj.x + lj.y * lj.y);
-  auto emit = [&](int64_t l, int64_t n, double zr, double zi) {
-    bk.put(l, p, n, lj.x * zr - lj.y * zi, lj.x * zi + lj.y * zr, am * sqrt(zr * zr + zi * zi));
+  auto emit = [&](int64_t l, int64_t n, auto value) {
+    bk.put(l, n, [&] {
+      const double2 z = value();
+      const double am = sqrt(lj.x * lj.x + lj.y * lj.y);
+      return BTerm{p, (int32_t)n, lj.x * z.x - lj.y * z.y, lj.x * z.y + lj.y * z.x, am * (fabs(z.x) + fabs(z.y))};
+    });
   };
   z_fiber_slice(B, j, (int)(it % S), emit);
 }
@@ -191,7 +207,12 @@ __global__ void k_q_pair_bucket(BasisView B, const double* h, const int64_t* hli
   if (it >= nh * S) return;
   const int64_t m = hlist[it / S];
   const double hm = h[m];
-  auto emit = [&](int64_t n, int64_t s, double f) { bk.put(s, -1, n, hm * f, 0.0, fabs(hm * f)); };
+  auto emit = [&](int64_t n, int64_t s, auto value) {
+    bk.put(s, n, [&] {
+      const double q = hm * value();
+      return BTerm{-1, (int32_t)n, q, 0.0, fabs(q)};
+    });
+  };
   f_fiber_slice(B, m, (int)(it % S), emit);
 }
 
@@ -205,9 +226,11 @@ __global__ void k_q_pair_bucket(BasisView B, const double* h, const int64_t* hli
 //   H_xy = [x >= 1] x_x lc_x + sum_{x < nu < y} x_nu c_nu + x_y (c_y + lc_y)
 //          + 2 sum_{nu > y} x_nu c_nu,
 // and d(D_nu, D_lam, D_mu) = 2 sum_k delta_k(nu) delta_k(lam) delta_k(mu).
-// One thread per (source, x) walks y upward keeping the running sum over
-// x < nu < y, so every sum holds exactly the terms of its edge; each term
-// carries the sum of the magnitudes of its parts.
+// One warp per (source, x) takes 32 consecutive y at a time: the sums over
+// x < nu < y are a prefix over the window and the windows before it, so every
+// sum holds exactly the terms of its edge; each term carries the sum of the
+// magnitudes of its parts.  Windows that no bucket wants only add their terms
+// lane by lane.  (One thread walking all y took 560 us a pass at N = 400.)
 
 // Diagonal components of every channel: dl[p N + nu] (complex), hasD[p].
 __global__ void k_dscatter(const BasisView B, int nP, const int64_t* lp_ptr, const int64_t* lp_idx,
@@ -223,50 +246,88 @@ __global__ void k_dscatter(const BasisView B, int nP, const int64_t* lp_ptr, con
   hasD[p] = 1;
 }
 
-// suf[p N + y] = sum_{nu > y} x_nu c_nu and sufm the same over |x_nu| c_nu.
-__global__ void k_dsuffix(const BasisView B, int nP, const double2* dl, const int* hasD, double2* suf, double* sufm) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nP || !hasD[p]) return;
-  const int N = B.N;
+// suf[p N + y] = sum_{nu > y} x_nu c_nu and sufm the same over |x_nu| c_nu; one
+// block per channel, each thread a contiguous run of nu.
+__global__ void __launch_bounds__(kSuffixThreads) k_dsuffix(const BasisView B, const double2* dl, const int* hasD,
+                                                            double2* suf, double* sufm) {
+  __shared__ double sh[kSuffixThreads / 32];
+  const int p = blockIdx.x, N = B.N;
+  if (!hasD[p]) return;
   const double2* x = dl + (int64_t)p * N;
+  const int per = (N + kSuffixThreads - 1) / kSuffixThreads, k0 = min((int)threadIdx.x * per, N),
+            k1 = min(k0 + per, N);
   double2 r = make_double2(0.0, 0.0);
   double rm = 0.0;
-  for (int y = N - 1; y >= 0; --y) {
+  auto add = [&](int y) {
+    const double c = ld_c(B, y);
+    r.x += x[y].x * c;
+    r.y += x[y].y * c;
+    rm += sqrt(x[y].x * x[y].x + x[y].y * x[y].y) * c;
+  };
+  for (int y = k1 - 1; y >= max(k0, 1); --y) add(y);
+  r.x = block_suffix(r.x, sh);
+  r.y = block_suffix(r.y, sh);
+  rm = block_suffix(rm, sh);
+  for (int y = k1 - 1; y >= k0; --y) {
     suf[(int64_t)p * N + y] = r;
     sufm[(int64_t)p * N + y] = rm;
-    if (y >= 1) {
-      const double c = ld_c(B, y);
-      r.x += x[y].x * c;
-      r.y += x[y].y * c;
-      rm += sqrt(x[y].x * x[y].x + x[y].y * x[y].y) * c;
-    }
+    if (y >= 1) add(y);
   }
 }
+
+// A sum over x < nu < y of one warp's windows: `acc` holds the lane's share of
+// the windows passed.  before(t) is the sum up to the lane's y, t its own term.
+struct WindowSum {
+  double acc = 0.0;
+  __device__ __forceinline__ void pass(double t) { acc += t; }
+  __device__ __forceinline__ double before(double t, int lane) {
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    double in = lane == 0 ? acc + t : t;  // inclusive prefix
+    for (int o = 1; o < 32; o <<= 1) {
+      const double u = __shfl_up_sync(0xffffffffu, in, o);
+      if (lane >= o) in += u;
+    }
+    const double ex = __shfl_up_sync(0xffffffffu, in, 1), r = lane == 0 ? acc : ex;
+    acc = lane == 31 ? in : 0.0;
+    return r;
+  }
+};
 
 // W and U terms of the diagonal components of channel p on edge (x, y):
 //   W(l = S, s = J) = conj(G),  W(l = J, s = S) = -conj(G),
 //   U(S, J) = G,  U(J, S) = -G,  U(S, S) = U(J, J) = i H.
 // mode 0: W terms, mode 1: U terms.
-__global__ void k_dpart_bucket(const BasisView B, int nP, const double2* dl, const int* hasD, const double2* suf,
-                               const double* sufm, int mode, Bucketer bk) {
-  const int N = B.N;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_dpart_bucket(const BasisView B, int nP, const double2* dl, const int* hasD,
+                                                      const double2* suf, const double* sufm, int mode, Bucketer bk) {
+  const int N = B.N, lane = threadIdx.x & 31;
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (t >= (int64_t)nP * N) return;
   const int p = (int)(t / N), x = (int)(t % N);
   if (!hasD[p]) return;
   const double2* dx = dl + (int64_t)p * N;
   const double2 head = x >= 1 ? make_double2(dx[x].x * ld_lc(B, x), dx[x].y * ld_lc(B, x)) : make_double2(0.0, 0.0);
   const double headm = x >= 1 ? sqrt(dx[x].x * dx[x].x + dx[x].y * dx[x].y) * fabs(ld_lc(B, x)) : 0.0;
-  double2 run = make_double2(0.0, 0.0);
-  double runm = 0.0;
+  WindowSum sr, si, sm;
   const int64_t P = B.P;
-  for (int y = x + 1; y < N; ++y) {
-    const double cy = ld_c(B, y), lcy = ld_lc(B, y);
-    const double2 xy = dx[y];
+  for (int y0 = x + 1; y0 < N; y0 += 32) {
+    const int y = y0 + lane;
+    const bool in = y < N;
+    const double cy = in ? ld_c(B, y) : 0.0, lcy = in ? ld_lc(B, y) : 0.0;
+    const double2 xy = in ? dx[y] : make_double2(0.0, 0.0);
     const double ay = sqrt(xy.x * xy.x + xy.y * xy.y);
+    const int64_t e = in ? pair_index(N, x, y) : 0, eS = e, eJ = P + e;
+    const bool want = in && (bk.wants(eS) || bk.wants(eJ));
+    if (!__any_sync(0xffffffffu, want)) {
+      sr.pass(xy.x * cy);
+      si.pass(xy.y * cy);
+      sm.pass(ay * cy);
+      continue;
+    }
+    const double2 run = make_double2(sr.before(xy.x * cy, lane), si.before(xy.y * cy, lane));
+    const double runm = sm.before(ay * cy, lane);
+    if (!want) continue;
     const double2 G = make_double2(head.x + run.x + xy.x * (cy - lcy), head.y + run.y + xy.y * (cy - lcy));
     const double Gm = headm + runm + ay * (cy - lcy);
-    const int64_t e = pair_index(N, x, y), eS = e, eJ = P + e;
     if (mode == 0) {
       if (Gm > 0.0) {
         bk.put(eJ, p, eS, G.x, -G.y, Gm);
@@ -285,11 +346,6 @@ __global__ void k_dpart_bucket(const BasisView B, int nP, const double2* dl, con
         bk.put(eS, p, eS, -H_im, H_re, Hm);
         bk.put(eJ, p, eJ, -H_im, H_re, Hm);
       }
-    }
-    if (y < N - 1) {  // x < nu < y' for the next y' = y + 1
-      run.x += xy.x * cy;
-      run.y += xy.y * cy;
-      runm += ay * cy;
     }
   }
 }
@@ -326,10 +382,7 @@ __global__ void k_udd_bucket(const BasisView B, int nP, const double2* dl, const
 
 // Q terms of the diagonal coefficients h_{D_lam}: only (S_xy, J_xy) and
 // (J_xy, S_xy), q_{S J} = sum_lam h_{D_lam} f(D_lam, J_xy, S_xy) = -G_xy[h]
-// and q_{J S} = -q_{S J}.  One warp per x: the lanes take 32 consecutive y
-// at a time, and the sums over x < lam < y are a warp prefix scan of
-// h_lam c_lam (and of |h_lam| c_lam) over that window plus the window's
-// carry, so each holds exactly the terms of its edge.
+// and q_{J S} = -q_{S J}.  One warp per x, in windows as above.
 __global__ void k_q_diag_bucket(BasisView B, const double* h, Bucketer bk) {
   const int N = B.N;
   const int x = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
@@ -338,38 +391,27 @@ __global__ void k_q_diag_bucket(BasisView B, const double* h, Bucketer bk) {
   const double* hd = h + 2 * B.P - 1;  // hd[nu] = h_{D_nu}
   const double head = x >= 1 ? hd[x] * ld_lc(B, x) : 0.0;
   const double headm = x >= 1 ? fabs(hd[x] * ld_lc(B, x)) : 0.0;
-  double carry = 0.0, carrym = 0.0;  // sums over x < lam < (the window's first y)
+  WindowSum sr, sm;
   for (int y0 = x + 1; y0 < N; y0 += 32) {
     const int y = y0 + lane;
     const bool in = y < N;
     const double cy = in ? ld_c(B, y) : 0.0, lcy = in ? ld_lc(B, y) : 0.0, hy = in ? hd[y] : 0.0;
-    double t = hy * cy, tm = fabs(hy) * cy;  // the term lam = y, for the larger y
-    double it = t, itm = tm;                  // inclusive prefix over the window
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double u = __shfl_up_sync(0xffffffffu, it, o), um = __shfl_up_sync(0xffffffffu, itm, o);
-      if (lane >= o) {
-        it += u;
-        itm += um;
-      }
+    const double t = hy * cy, tm = fabs(t);  // the term lam = y, for the larger y
+    const int64_t e = in ? pair_index(N, x, y) : 0;
+    const bool want = in && (bk.wants(e) || bk.wants(B.P + e));
+    if (!__any_sync(0xffffffffu, want)) {
+      sr.pass(t);
+      sm.pass(tm);
+      continue;
     }
-    double ex = __shfl_up_sync(0xffffffffu, it, 1), exm = __shfl_up_sync(0xffffffffu, itm, 1);
-    if (lane == 0) {
-      ex = 0.0;
-      exm = 0.0;
+    const double run = sr.before(t, lane), runm = sm.before(tm, lane);  // x < lam < y
+    if (!want) continue;
+    const double G = head + run + hy * (cy - lcy);
+    const double Gm = headm + runm + fabs(hy) * (cy - lcy);
+    if (Gm > 0.0) {
+      bk.put(e, -1, B.P + e, -G, 0.0, Gm);
+      bk.put(B.P + e, -1, e, G, 0.0, Gm);
     }
-    const double run = carry + ex, runm = carrym + exm;  // x < lam < y
-    if (in) {
-      const double G = head + run + hy * (cy - lcy);
-      const double Gm = headm + runm + fabs(hy) * (cy - lcy);
-      if (Gm > 0.0) {
-        const int64_t e = pair_index(N, x, y);
-        bk.put(e, -1, B.P + e, -G, 0.0, Gm);
-        bk.put(B.P + e, -1, e, G, 0.0, Gm);
-      }
-    }
-    carry += __shfl_sync(0xffffffffu, it, 31);
-    carrym += __shfl_sync(0xffffffffu, itm, 31);
   }
 }
 
@@ -383,10 +425,12 @@ __global__ void k_k_lowrank(BasisView B, int nP, const int64_t* lp_ptr, const do
   if (t >= n * n) return;
   const int64_t u = base + t / n, w = base + t % n;
   const int64_t j = lp_idx[u], k = lp_idx[w];
+  const Elem ej = decode(B, j), ek = decode(B, k);
+  // two edges without a common vertex meet in no structure constant (most pairs, so before any FP64)
+  if (ej.kind != kD && ek.kind != kD && ej.a != ek.a && ej.a != ek.b && ej.b != ek.a && ej.b != ek.b) return;
   const double2 lj = lp_val[u], lk = lp_val[w];
   const double aim = gamma[p] * (lj.y * lk.x - lj.x * lk.y);  // Im(l_j conj(l_k))
   if (aim == 0.0) return;
-  const Elem ej = decode(B, j), ek = decode(B, k);
   const double inv = -1.0 / (double)B.N;
   auto add = [&](const Elem& es, int64_t s) {
     const double f = f_value(B, ej, ek, es);
@@ -418,6 +462,7 @@ __global__ void k_k_lowrank(BasisView B, int nP, const int64_t* lp_ptr, const do
 // tile scans with their offsets.  A tile is 256 threads x 8 counts.
 constexpr int kScanThreads = 256, kScanItems = 8, kScanTile = kScanThreads * kScanItems;
 
+template <int T = kScanThreads>
 __device__ __forceinline__ int64_t block_excl_scan(int64_t x, int64_t* warp_tot, int64_t& total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int64_t inc = x;
@@ -429,16 +474,16 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t x, int64_t* warp_tot,
   if (lane == 31) warp_tot[wid] = inc;
   __syncthreads();
   if (wid == 0) {
-    int64_t w = lane < kScanThreads / 32 ? warp_tot[lane] : 0;
+    int64_t w = lane < T / 32 ? warp_tot[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int64_t t = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += t;
     }
-    if (lane < kScanThreads / 32) warp_tot[lane] = w;  // inclusive warp totals
+    if (lane < T / 32) warp_tot[lane] = w;  // inclusive warp totals
   }
   __syncthreads();
-  total = warp_tot[kScanThreads / 32 - 1];
+  total = warp_tot[T / 32 - 1];
   const int64_t before = wid > 0 ? warp_tot[wid - 1] : 0;
   const int64_t r = before + inc - x;
   __syncthreads();
@@ -490,8 +535,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(int64_t* tile_sum, in
 constexpr int kRowCap = 512;          // hash slots of one warp (rows up to 256 terms)
 constexpr int kRowBound = 256;        // terms above which a row takes the block path
 constexpr int kRowWarps = 4;
+constexpr int kMidBound = 1024;       // rows up to this many terms take a small table of the block path
 constexpr int kLongCap = 8192;        // hash slots of one block (long rows), per column partition
-constexpr int kLongThreads = 256;
+constexpr int kMidThreads = 256, kLongThreads = 1024;
+constexpr int kLongMinCap = 1024;
 constexpr int32_t kEmpty = -1;
 
 // The rows at hand: s = list[i], i < rows (list null: all rows).
@@ -583,8 +630,8 @@ struct WStage {
   int32_t p, pre;
 };
 
-// Exclusive prefix of x over the WIDTH threads (WIDTH = 32: one warp;
-// WIDTH = kLongThreads: the block, with a barrier); *total = the sum.
+// Exclusive prefix of x over the WIDTH threads (WIDTH = 32: one warp,
+// else the block, with a barrier); *total = the sum.
 template <int WIDTH>
 __device__ __forceinline__ int excl_prefix(int x, int* tot_s, int* total) {
   if (WIDTH == 32) {
@@ -599,7 +646,7 @@ __device__ __forceinline__ int excl_prefix(int x, int* tot_s, int* total) {
     return inc - x;
   } else {
     int64_t t64;
-    const int64_t r = block_excl_scan((int64_t)x, reinterpret_cast<int64_t*>(tot_s), t64);
+    const int64_t r = block_excl_scan<WIDTH>((int64_t)x, reinterpret_cast<int64_t*>(tot_s), t64);
     *total = (int)t64;
     return (int)r;
   }
@@ -737,10 +784,11 @@ __device__ __forceinline__ int warp_compact(int32_t* keys, double* val, double* 
   return run;
 }
 
-// Terms of every row (one warp per row): bound[s]; rows of more than
-// kRowBound terms go to the long list.
+// Terms of every row (one warp per row): bound[i] of row list[i]; rows of more than
+// kRowBound terms go to the long list, those of more than kMidBound from its end.
 __global__ void __launch_bounds__(kRowWarps * 32) k_row_terms(RowInputs I, unsigned long long* bound,
-                                                             int64_t* longlist, unsigned long long* nlong) {
+                                                             int64_t* longlist, unsigned long long* nmid,
+                                                             unsigned long long* nlong) {
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * kRowWarps + wid;
   if (i >= I.rows) return;
@@ -748,15 +796,16 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_row_terms(RowInputs I, unsig
   int64_t t = row_terms(I, s, lane, 32);
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) {
-    bound[s] = (unsigned long long)t;
-    if (t > kRowBound) longlist[atomicAdd(nlong, 1ull)] = s;
+    bound[i] = (unsigned long long)t;
+    if (t > kMidBound) longlist[I.rows - 1 - (int64_t)atomicAdd(nlong, 1ull)] = i;
+    else if (t > kRowBound) longlist[atomicAdd(nmid, 1ull)] = i;
   }
 }
 
 // One warp per row of at most kRowBound terms, in a table of the smallest
 // power of two >= 2 x terms slots (at least 64): accumulate the row once and
-// write its kept entries (unordered) to the row's scratch range (tmpoff[s],
-// room for bound[s] >= kept entries) and their number to rowcount[s].
+// write its kept entries (unordered) to the row's scratch range (tmpoff[i],
+// room for bound[i] >= kept entries) and their number to rowcount[s].
 __global__ void __launch_bounds__(kRowWarps * 32) k_rows_warp(RowInputs I, const unsigned long long* bound,
                                                              const int64_t* tmpoff, int32_t* tcol, double* tval,
                                                              unsigned long long* rowcount, int* status) {
@@ -767,7 +816,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_warp(RowInputs I, const
   const int64_t i = (int64_t)blockIdx.x * kRowWarps + wid;
   if (i >= I.rows) return;
   const int64_t s = I.list ? I.list[i] : i;
-  const unsigned long long tb = bound[s];
+  const unsigned long long tb = bound[i];
   if (tb > (unsigned long long)kRowBound) return;
   int cap = 64;
   while (cap < 2 * (int)tb) cap <<= 1;
@@ -785,55 +834,67 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows_warp(RowInputs I, const
   __syncwarp();
   const int k = warp_compact(keys, val, mag, cap, lane);
   for (int e = lane; e < k; e += 32) {
-    tcol[tmpoff[s] + e] = keys[e];
-    tval[tmpoff[s] + e] = val[e];
+    tcol[tmpoff[i] + e] = keys[e];
+    tval[tmpoff[i] + e] = val[e];
   }
   if (lane == 0) rowcount[s] = (unsigned long long)k;
 }
 
 // One block per long row.  The row's columns are split by the high bits of
 // their hash into the smallest power-of-two number of partitions with at
-// most kLongCap / 2 terms each on average; each partition is accumulated in
-// a table of kLongCap slots in shared memory and its kept entries appended
-// to the row's scratch range.  A partition with more distinct columns than
-// slots sets *status = 2.
-__global__ void __launch_bounds__(kLongThreads) k_rows_long(RowInputs I, const int64_t* longlist,
+// most maxcap / 2 terms each on average; each partition is accumulated in a
+// table in shared memory, of the smallest power of two >= 2 x terms slots up to
+// maxcap, and its kept entries are appended to the row's scratch range (in any
+// order).  A partition with more distinct columns than slots sets *status = 2.
+// Rows of at most kMidBound terms are launched with maxcap = 2 kMidBound, 40 KB:
+// five blocks an SM in place of one, and less to clear and to look through; the
+// others have an SM to themselves, so they take 32 warps (the additions to the
+// table are chains of atomics: 8800 rows of the ladder at N = 2000 in 1.8 ms, with
+// 8 warps 2.75 ms, all in one class 3.8 ms).
+template <int T>
+__global__ void __launch_bounds__(T) k_rows_long(RowInputs I, const int64_t* longlist, int maxcap,
                                                            const unsigned long long* bound, const int64_t* tmpoff,
                                                            int32_t* tcol, double* tval, unsigned long long* rowcount,
                                                            int* status) {
   extern __shared__ __align__(16) unsigned char lsm[];
+  __shared__ WStage ws[T];
+  __shared__ int64_t tot_s[T / 32];
+  __shared__ int total;
+  const int64_t i = longlist[blockIdx.x], s = I.list ? I.list[i] : i;
+  const unsigned long long tb = bound[i];
+  int nparts = 1, cap = kLongMinCap;
+  while ((unsigned long long)nparts * (maxcap / 2) < tb && nparts < (1 << 20)) nparts <<= 1;
+  while (cap < maxcap && (unsigned long long)cap < 2 * tb) cap <<= 1;
   double* val = reinterpret_cast<double*>(lsm);
-  double* mag = val + kLongCap;
-  int32_t* keys = reinterpret_cast<int32_t*>(mag + kLongCap);
-  __shared__ WStage ws[kLongThreads];
-  __shared__ int64_t tot_s[kLongThreads / 32];
-  __shared__ int kk;
-  const int64_t s = longlist[blockIdx.x];
-  int nparts = 1;
-  while ((unsigned long long)nparts * (kLongCap / 2) < bound[s] && nparts < (1 << 20)) nparts <<= 1;
-  int total = 0;
+  double* mag = val + cap;
+  int32_t* keys = reinterpret_cast<int32_t*>(mag + cap);
+  const int lane = threadIdx.x & 31;
+  const int64_t dst = tmpoff[i];
+  if (threadIdx.x == 0) total = 0;
   for (int part = 0; part < nparts; ++part) {
-    for (int a = threadIdx.x; a < kLongCap; a += kLongThreads) {
+    for (int a = threadIdx.x; a < cap; a += T) {
       keys[a] = kEmpty;
       val[a] = 0.0;
       mag[a] = 0.0;
     }
     __syncthreads();
-    const bool ok = row_accumulate<kLongThreads>(I, s, threadIdx.x, ws, reinterpret_cast<int*>(tot_s), keys, val, mag,
-                                                 kLongCap - 1, part, nparts);
+    const bool ok = row_accumulate<T>(I, s, threadIdx.x, ws, reinterpret_cast<int*>(tot_s), keys, val, mag,
+                                                 cap - 1, part, nparts);
     if (!ok) atomicExch(status, 2);
     __syncthreads();
-    if (threadIdx.x < 32) {  // compaction by warp 0
-      const int k = warp_compact(keys, val, mag, kLongCap, threadIdx.x);
-      if (threadIdx.x == 0) kk = k;
+    for (int a = threadIdx.x; a < cap; a += T) {  // cap is a multiple of the threads
+      const int32_t k = keys[a];
+      const double v = val[a];
+      const bool kp = kept(k, v, mag[a]);
+      const unsigned bal = __ballot_sync(0xffffffffu, kp);
+      int at = 0;
+      if (lane == 0 && bal) at = atomicAdd(&total, __popc(bal));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (kp) {
+        tcol[dst + at] = k;
+        tval[dst + at] = v;
+      }
     }
-    __syncthreads();
-    const int k = kk;
-    for (int e = threadIdx.x; e < k; e += kLongThreads) {
-      tcol[tmpoff[s] + total + e] = keys[e];
-      tval[tmpoff[s] + total + e] = val[e];
-    }
-    total += k;
     __syncthreads();
   }
   if (threadIdx.x == 0) rowcount[s] = (unsigned long long)total;
@@ -849,7 +910,7 @@ __global__ void __launch_bounds__(256) k_rows_copy(int64_t rows, const int64_t* 
   const int lane = threadIdx.x & 31;
   if (i >= rows) return;
   const int64_t s = list ? list[i] : i;
-  const int64_t src = tmpoff[s], dst = rowptr[s], k = rowptr[s + 1] - rowptr[s];
+  const int64_t src = tmpoff[i], dst = rowptr[s], k = rowptr[s + 1] - rowptr[s];
   for (int64_t q = lane; q < k; q += 32) {
     const int32_t kq = tcol[src + q];
     int64_t rank = 0;
@@ -870,7 +931,7 @@ namespace lbi {
 // cudaFree of the sizes here takes 0.1 to several ms and synchronizes the
 // device; the ladder at N = 2000 spent 10 of its 41 ms in them), the rest goes
 // back at the next synchronization, all of it with lb_host_release.
-constexpr uint64_t kScratchKeep = uint64_t(1) << 30;
+constexpr uint64_t kScratchKeep = uint64_t(2) << 30, kLargeScratch = uint64_t(1) << 29;
 
 cudaError_t scratch_pool(cudaMemPool_t* out) {
   static std::mutex mu;
@@ -918,12 +979,14 @@ struct Buf {
   explicit Buf(cudaStream_t s) : st(s) {}
   Buf(const Buf&) = delete;
   Buf& operator=(const Buf&) = delete;
-  ~Buf() {
+  ~Buf() { release(); }
+  void release() {  // behind the work queued on st
     if (p && large) cudaFree(p);
     else if (p) cudaFreeAsync(p, st);
+    p = nullptr;
   }
   cudaError_t alloc(size_t n) {
-    if (n > kScratchKeep / 2) {
+    if (n > kLargeScratch) {
       large = true;
       return cudaMalloc(&p, n);
     }
@@ -975,18 +1038,27 @@ struct Buckets {
   explicit Buckets(cudaStream_t st) : cnt(st), off(st), terms(st) {}
 };
 
-// Count with `emit(bucketer)`, scan, reset the cursors, fill with `emit`.
+// Count with `emit(bucketer)` and scan; the total goes to the host's b.total
+// with the next synchronization.
 template <class Emit>
-static cudaError_t build_buckets(int64_t M, Buckets& b, const uint8_t* keep, uint8_t* mark, Emit emit,
+static cudaError_t count_buckets(int64_t M, Buckets& b, const uint8_t* keep, uint8_t* mark, Emit emit,
                                  cudaStream_t st) {
   CK(b.cnt.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
   CK(b.off.alloc(sizeof(int64_t) * (size_t)(M + 1)));
   CK(cudaMemsetAsync(b.cnt.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
   CK(emit(Bucketer{b.cnt.as<unsigned long long>(), nullptr, nullptr, keep, mark}));
-  CK(scan_counts(b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), M, &b.total, st));
+  CK(scan_device(b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), M, st));
+  return cudaMemcpyAsync(&b.total, b.off.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+}
+
+// Reset the cursors, fill with `emit`.
+template <class Emit>
+static cudaError_t fill_buckets(int64_t M, Buckets& b, const uint8_t* keep, Emit emit, cudaStream_t st) {
   CK(b.terms.alloc(sizeof(BTerm) * (size_t)b.total));
+  if (b.total == 0) return cudaSuccess;
   CK(cudaMemsetAsync(b.cnt.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
-  if (b.total > 0) CK(emit(Bucketer{b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), b.terms.as<BTerm>(), keep, nullptr}));
+  CK(emit(Bucketer{b.cnt.as<unsigned long long>(), b.off.as<int64_t>(), b.terms.as<BTerm>(), keep, nullptr}));
+  b.cnt.release();
   return cudaSuccess;
 }
 
@@ -1012,52 +1084,61 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   CK(cudaMemsetAsync(hasD.p, 0, sizeof(int) * (size_t)(nP > 0 ? nP : 1), st));
   if (nu > 0) {
     k_dscatter<<<nb(nu, 256), 256, 0, st>>>(B, nP, dp, lp_idx, lp_val, nu, dl.as<double2>(), hasD.as<int>());
-    k_dsuffix<<<nb(nP, 128), 128, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
-                                           sufm.as<double>());
+    k_dsuffix<<<nP, kSuffixThreads, 0, st>>>(B, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
+                                             sufm.as<double>());
     note_launch(2);
   }
   const int64_t ndp = (int64_t)nP * N, ndd = (int64_t)nP * (N - 1) * (N - 1);
   const int S = fiber_slices(N);
-  // ---- rows in closed form: their counts, and the list of the rows that are left.  Below 64 levels too many rows
-  // are near the diagonal for the extra launches to pay; more channels than four have no tables
-  const bool bulk = N >= 64 && nP <= 4 && csr_bulk_bytes(N, nP) <= kScratchKeep / 2;
-  Buf bmem(st), rowc(st), list(st), need(st), bctr(st);  // bctr: [0] join terms, [1] rows left
+  // ---- the nonzero pair coefficients of h, and the rows in closed form with the list of the rows that are left.
+  // Below 128 levels too many rows are near the diagonal for the extra launches to pay (against the join alone:
+  // ladder N = 70 622 / 567 us, N = 100 638 / 613, N = 140 668 / 688; N = 400 dimer 1.2 / 3.7 ms); more channels than
+  // four have no tables
+  const bool bulk = N >= 128 && nP <= 4 && csr_bulk_bytes(N, nP) <= kLargeScratch;
+  Buf bmem(st), rowc(st), list(st), need(st), bctr(st), hlist(st);  // bctr: join terms, rows left, nonzeros of h
   CsrBulk cb{};
   CK(rowc.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
-  unsigned long long hb[2] = {0, (unsigned long long)M};
+  CK(bctr.alloc(sizeof(unsigned long long) * 3));
+  CK(cudaMemsetAsync(bctr.p, 0, sizeof(unsigned long long) * 3, st));
+  unsigned long long* bc = bctr.as<unsigned long long>();
+  if (h) {
+    CK(hlist.alloc(sizeof(int64_t) * (size_t)(2 * B.P)));
+    k_h_nonzero<<<nb(2 * B.P, 256), 256, 0, st>>>(2 * B.P, h, hlist.as<int64_t>(), bc + 2);
+    note_launch(1);
+  }
   if (bulk) {
     CK(bmem.alloc(csr_bulk_bytes(N, nP)));
     CK(list.alloc(sizeof(int64_t) * (size_t)M));
     CK(need.alloc((size_t)M));
-    CK(bctr.alloc(sizeof(hb)));
-    CK(cudaMemsetAsync(bctr.p, 0, sizeof(hb), st));
     CK(cudaMemsetAsync(need.p, 0, (size_t)M, st));
     CK(cudaMemsetAsync(rowc.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
     cb = csr_bulk_carve(bmem.p, N, nP, dgamma.as<double>());
-    unsigned long long* bc = bctr.as<unsigned long long>();
     CK(csr_bulk_count(B, cb, nP, dp, lp_idx, lp_val, nu, dl.as<double2>(), hasD.as<int>(), h,
                       rowc.as<unsigned long long>(), bc, list.as<int64_t>(), bc + 1, st));
+  }
+  unsigned long long hb[3] = {0, 0, 0};
+  if (bulk || h) {
     CK(cudaMemcpyAsync(hb, bctr.p, sizeof(hb), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
   }
-  const uint8_t* slow = bulk ? cb.slow : nullptr;
-  const int64_t rows = (int64_t)hb[1];
+  const uint8_t *slow = bulk ? cb.slow : nullptr, *needed = bulk ? need.as<uint8_t>() : nullptr;
+  const int64_t rows = bulk ? (int64_t)hb[1] : M, nh = (int64_t)hb[2];
   // ---- W (by column s), U (by row l), Q (by row s)
   Buckets W(st), U(st), Q(st);
-  CK(build_buckets(M, W, slow, bulk ? need.as<uint8_t>() : nullptr, [&](Bucketer bk) {
+  auto emit_w = [&](Bucketer bk) {
     if (nu > 0) {
       k_w_bucket<<<nb(nu * S, 256), 256, 0, st>>>(B, nP, dp, lp_idx, lp_val, nu, bk);
-      k_dpart_bucket<<<nb(ndp, 128), 128, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
-                                                   sufm.as<double>(), 0, bk);
+      k_dpart_bucket<<<nb(ndp * 32, 256), 256, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
+                                                        sufm.as<double>(), 0, bk);
       note_launch(2);
     }
     return cudaGetLastError();
-  }, st));
-  CK(build_buckets(M, U, bulk ? need.as<uint8_t>() : nullptr, nullptr, [&](Bucketer bk) {
+  };
+  auto emit_u = [&](Bucketer bk) {
     if (nu > 0) {
       k_u_bucket<<<nb(nu * S, 256), 256, 0, st>>>(B, nP, dp, lp_idx, lp_val, nu, bk);
-      k_dpart_bucket<<<nb(ndp, 128), 128, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
-                                                   sufm.as<double>(), 1, bk);
+      k_dpart_bucket<<<nb(ndp * 32, 256), 256, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
+                                                        sufm.as<double>(), 1, bk);
       note_launch(2);
       if (ndd > 0) {
         k_udd_bucket<<<nb(ndd, 256), 256, 0, st>>>(B, nP, dl.as<double2>(), hasD.as<int>(), suf.as<double2>(),
@@ -1066,48 +1147,43 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
       }
     }
     return cudaGetLastError();
-  }, st));
-  if (h) {
-    Buf hlist(st), hcount(st);
-    CK(hlist.alloc(sizeof(int64_t) * (size_t)(2 * B.P)));
-    CK(hcount.alloc(sizeof(unsigned long long)));
-    CK(cudaMemsetAsync(hcount.p, 0, sizeof(unsigned long long), st));
-    k_h_nonzero<<<nb(2 * B.P, 256), 256, 0, st>>>(2 * B.P, h, hlist.as<int64_t>(), hcount.as<unsigned long long>());
-    note_launch(1);
-    unsigned long long nh = 0;
-    CK(cudaMemcpyAsync(&nh, hcount.p, sizeof(nh), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    CK(build_buckets(M, Q, slow, nullptr, [&](Bucketer bk) {
-      if (nh > 0) {
-        k_q_pair_bucket<<<nb((int64_t)nh * S, 256), 256, 0, st>>>(B, h, hlist.as<int64_t>(), (int64_t)nh, bk);
-        note_launch(1);
-      }
-      k_q_diag_bucket<<<nb((int64_t)N * 32, 256), 256, 0, st>>>(B, h, bk);
+  };
+  auto emit_q = [&](Bucketer bk) {
+    if (nh > 0) {
+      k_q_pair_bucket<<<nb(nh * S, 256), 256, 0, st>>>(B, h, hlist.as<int64_t>(), nh, bk);
       note_launch(1);
-      return cudaGetLastError();
-    }, st));
-  }
+    }
+    k_q_diag_bucket<<<nb((int64_t)N * 32, 256), 256, 0, st>>>(B, h, bk);
+    note_launch(1);
+    return cudaGetLastError();
+  };
+  CK(count_buckets(M, W, slow, bulk ? need.as<uint8_t>() : nullptr, emit_w, st));
+  CK(count_buckets(M, U, needed, nullptr, emit_u, st));
+  if (h) CK(count_buckets(M, Q, slow, nullptr, emit_q, st));
+  CK(cudaStreamSynchronize(st));
+  CK(fill_buckets(M, W, slow, emit_w, st));
+  CK(fill_buckets(M, U, needed, emit_u, st));
+  if (h) CK(fill_buckets(M, Q, slow, emit_q, st));
+  hlist.release();
   // ---- rows: term bounds, one accumulation into scratch ranges, CSR
-  RowInputs I{rows, bulk ? list.as<int64_t>() : nullptr, dgamma.as<double>(), W.off.as<int64_t>(), U.off.as<int64_t>(), h ? Q.off.as<int64_t>() : nullptr,
-              W.terms.as<BTerm>(), U.terms.as<BTerm>(), h ? Q.terms.as<BTerm>() : nullptr};
-  Buf bound(st), tmpoff(st), longlist(st), ctr(st);  // ctr: [0] long rows, [1] status
-  CK(bound.alloc(sizeof(unsigned long long) * (size_t)(M + 1)));
-  CK(tmpoff.alloc(sizeof(int64_t) * (size_t)(M + 1)));
-  CK(longlist.alloc(sizeof(int64_t) * (size_t)M));
-  CK(ctr.alloc(sizeof(unsigned long long) * 2));
-  CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned long long) * 2, st));
-  if (bulk) CK(cudaMemsetAsync(bound.p, 0, sizeof(unsigned long long) * (size_t)(M + 1), st));
+  RowInputs I{rows, bulk ? list.as<int64_t>() : nullptr, dgamma.as<double>(), W.off.as<int64_t>(),
+              U.off.as<int64_t>(), h ? Q.off.as<int64_t>() : nullptr, W.terms.as<BTerm>(), U.terms.as<BTerm>(), h ? Q.terms.as<BTerm>() : nullptr};
+  Buf bound(st), tmpoff(st), longlist(st), ctr(st);  // ctr: middle rows, long rows, status
+  CK(bound.alloc(sizeof(unsigned long long) * (size_t)(rows + 1)));
+  CK(tmpoff.alloc(sizeof(int64_t) * (size_t)(rows + 1)));
+  CK(longlist.alloc(sizeof(int64_t) * (size_t)rows));
+  CK(ctr.alloc(sizeof(unsigned long long) * 3));
+  CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned long long) * 3, st));
   unsigned long long* c = ctr.as<unsigned long long>();
-  int* status = reinterpret_cast<int*>(c + 1);
+  int* status = reinterpret_cast<int*>(c + 2);
   const unsigned rgrid = std::max(nb(rows, kRowWarps), 1u);
-  k_row_terms<<<rgrid, kRowWarps * 32, 0, st>>>(I, bound.as<unsigned long long>(), longlist.as<int64_t>(), c);
+  k_row_terms<<<rgrid, kRowWarps * 32, 0, st>>>(I, bound.as<unsigned long long>(), longlist.as<int64_t>(), c, c + 1);
   note_launch(1);
   int64_t nterms = 0;
-  CK(scan_counts(bound.as<unsigned long long>(), tmpoff.as<int64_t>(), M, &nterms, st));
-  unsigned long long hc[2];
+  unsigned long long hc[3];
   CK(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  const int64_t nlong = (int64_t)hc[0];
+  CK(scan_counts(bound.as<unsigned long long>(), tmpoff.as<int64_t>(), rows, &nterms, st));
+  const int64_t nmid = (int64_t)hc[0], nlong = (int64_t)hc[1];
   Buf tcol(st), tval(st);
   CK(tcol.alloc(sizeof(int32_t) * (size_t)(nterms + 1)));
   CK(tval.alloc(sizeof(double) * (size_t)(nterms + 1)));
@@ -1115,28 +1191,30 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
                                                 tcol.as<int32_t>(), tval.as<double>(), rowc.as<unsigned long long>(),
                                                 status);
   note_launch(1);
-  if (nlong > 0) {
-    const size_t lsmem = (sizeof(double) * 2 + sizeof(int32_t)) * (size_t)kLongCap;
-    CK(cudaFuncSetAttribute(k_rows_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem));
-    k_rows_long<<<(unsigned)nlong, kLongThreads, lsmem, st>>>(I, longlist.as<int64_t>(),
-                                                             bound.as<unsigned long long>(), tmpoff.as<int64_t>(),
-                                                             tcol.as<int32_t>(), tval.as<double>(),
-                                                             rowc.as<unsigned long long>(), status);
+  auto rows_long = [&](auto kernel, int threads, int64_t n, const int64_t* ll, int cap) {
+    if (n == 0) return cudaSuccess;
+    const size_t smem = (sizeof(double) * 2 + sizeof(int32_t)) * (size_t)cap;
+    CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<(unsigned)n, threads, smem, st>>>(I, ll, cap, bound.as<unsigned long long>(), tmpoff.as<int64_t>(),
+                                               tcol.as<int32_t>(), tval.as<double>(), rowc.as<unsigned long long>(),
+                                               status);
     note_launch(1);
-  }
+    return cudaGetLastError();
+  };
+  CK(rows_long(k_rows_long<kLongThreads>, kLongThreads, nlong, longlist.as<int64_t>() + (rows - nlong), kLongCap));
+  CK(rows_long(k_rows_long<kMidThreads>, kMidThreads, nmid, longlist.as<int64_t>(), 2 * kMidBound));
   Buf rowptr(st);
   CK(rowptr.alloc(sizeof(int64_t) * (size_t)(M + 1)));
   int64_t nnz = 0;
-  CK(scan_counts(rowc.as<unsigned long long>(), rowptr.as<int64_t>(), M, &nnz, st));
   CK(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (hc[1] != 0) return cudaErrorNotSupported;  // a row has more than kLongCap distinct columns
+  CK(scan_counts(rowc.as<unsigned long long>(), rowptr.as<int64_t>(), M, &nnz, st));
+  if (hc[2] != 0) return cudaErrorNotSupported;  // a row has more than kLongCap distinct columns
   Buf col(st), val(st), K(st);
   CK(col.alloc(sizeof(int32_t) * (size_t)(nnz + 1)));
   CK(val.alloc(sizeof(double) * (size_t)(nnz + 1)));
   CK(K.alloc(sizeof(double) * (size_t)M));
-  k_rows_copy<<<std::max(nb(rows, 8), 1u), 256, 0, st>>>(rows, I.list, tmpoff.as<int64_t>(), tcol.as<int32_t>(), tval.as<double>(),
-                                        rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>());
+  k_rows_copy<<<std::max(nb(rows, 8), 1u), 256, 0, st>>>(rows, I.list, tmpoff.as<int64_t>(), tcol.as<int32_t>(),
+                                                         tval.as<double>(), rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>());
   note_launch(1);
   if (bulk) CK(csr_bulk_fill(B, cb, nP, rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>(), st));
   // ---- K

@@ -22,12 +22,15 @@
 // neither, and a row with an entry in between goes the general way.
 //
 // What bounds it: the FP64 pipe (k_bulk_rows runs once over the pairs to count
-// and once to fill, 1.4 and 1.2 ms at N = 2000).  Whole assembly, with the
-// scratch kept between calls: ladder N = 2000 40.9 -> 13.7 ms, N = 500 4.6 ->
-// 1.5 ms, N = 100 1.20 -> 0.73 ms; dimer N = 400 6.2 -> 3.7 ms.
+// and once to fill, 1.0 and 0.65 ms at N = 2000, 1.4 and 1.25 ms with complex
+// products and FP64 comparisons throughout).  Whole assembly, with the scratch
+// kept between calls and the join's passes free of FP64 work for entries that
+// are only counted or dropped: ladder N = 2000 40.9 -> 7.1 ms, N = 1000 12.0 ->
+// 2.0 ms; dimer N = 400 6.2 -> 1.2 ms.
 #include <algorithm>
 
 #include "lb_internal.h"
+#include "lb_rowsum.cuh"
 
 namespace {
 
@@ -104,22 +107,24 @@ __device__ double block_max(double x, double* sh) {
 
 // Diagonals, block p < nP: channel p, block nP: H.
 //   x_kk = sum_{nu > k} x_nu c_nu + x_k lc_k   (x_0 = 0)
-// Each thread sums a contiguous run of nu; the runs' suffixes come from shared
-// memory.  gd[p] = 4 sum |x_nu| c_nu + 2 max |x_nu lc_nu|: above every diagonal
-// sum of an edge, summed by magnitude.
-__global__ void __launch_bounds__(256) k_bulk_diag(BasisView B, int nP, const double2* dl, const int* hasD,
-                                                   const double* h, CsrBulk b) {
-  __shared__ double sh[8];
-  __shared__ double run[256][2];
+// Each thread sums a contiguous run of nu; the sums of the runs behind it come
+// from the block.  gd[p] = 4 sum |x_nu| c_nu + 2 max |x_nu lc_nu|: above every
+// diagonal sum of an edge, summed by magnitude.  npd[p N + k]: the nonzero ones
+// of D_1 .. D_k.
+__global__ void __launch_bounds__(kSuffixThreads) k_bulk_diag(BasisView B, int nP, const double2* dl, const int* hasD,
+                                                              const double* h, CsrBulk b) {
+  __shared__ double sh[kSuffixThreads / 32];
   const int p = blockIdx.x, N = B.N, t = threadIdx.x;
   const bool isH = p == nP;
   const int64_t nn = (int64_t)N * N;
   auto at = [&](int nu) {  // component of D_nu
+    if (nu < 1) return make_double2(0.0, 0.0);
     if (isH) return make_double2(h ? h[2 * B.P - 1 + nu] : 0.0, 0.0);
     return hasD[p] ? dl[(int64_t)p * N + nu] : make_double2(0.0, 0.0);
   };
-  const int per = (N + 255) / 256, k0 = t * per, k1 = min(k0 + per, N);
+  const int per = (N + kSuffixThreads - 1) / kSuffixThreads, k0 = min(t * per, N), k1 = min(k0 + per, N);
   double sr = 0.0, si = 0.0, sm = 0.0, mlc = 0.0;
+  int n = 0;
   for (int nu = max(k0, 1); nu < k1; ++nu) {
     const double2 x = at(nu);
     const double c = ld_c(B, nu), m = sqrt(x.x * x.x + x.y * x.y);
@@ -127,25 +132,25 @@ __global__ void __launch_bounds__(256) k_bulk_diag(BasisView B, int nP, const do
     si += x.y * c;
     sm += m * c;
     mlc = fmax(mlc, m * fabs(ld_lc(B, nu)));
+    n += x.x != 0.0 || x.y != 0.0;
   }
-  run[t][0] = sr;
-  run[t][1] = si;
   const double gsum = block_sum(sm, sh), glc = block_max(mlc, sh);
+  double ar = block_suffix(sr, sh), ai = block_suffix(si, sh);  // sum over nu > the element at hand
+  const int behind = block_suffix(n, reinterpret_cast<int*>(sh));
+  __shared__ int total;
+  if (t == 0) total = n + behind;
   __syncthreads();
-  double ar = 0.0, ai = 0.0;  // sum over nu > the element at hand
-  if (gsum > 0.0)
-    for (int q = t + 1; q < 256; ++q) {
-      ar += run[q][0];
-      ai += run[q][1];
-    }
+  int upto = total - behind;  // nonzero ones of D_1 .. D_k
   for (int k = k1 - 1; k >= k0; --k) {
-    const double2 x = k > 0 ? at(k) : make_double2(0.0, 0.0);
+    const double2 x = at(k);
     const double lc = k > 0 ? ld_lc(B, k) : 0.0, c = k > 0 ? ld_c(B, k) : 0.0;
     const double2 d = make_double2(ar + x.x * lc, ai + x.y * lc);
     if (isH) b.hdiag[k] = d.x;
     else b.L[p * nn + (int64_t)k * N + k] = d;
     ar += x.x * c;
     ai += x.y * c;
+    b.npd[(int64_t)p * N + k] = upto;
+    upto -= x.x != 0.0 || x.y != 0.0;
   }
   if (t == 0) b.gd[p] = 4.0 * gsum + 2.0 * glc;
 }
@@ -363,7 +368,9 @@ __global__ void __launch_bounds__(128) k_bulk_vertex(BasisView B, int nP, const 
       b.ucol[at] = a;
       b.G[at] = g[q];
       for (int p = 0; p < nP; ++p) {
-        b.Lu[((int64_t)p * N + c) * kMaxDeg + rank] = b.L[p * nn + (int64_t)c * N + a];
+        const double2 x = b.L[p * nn + (int64_t)c * N + a];
+        b.Lu[((int64_t)p * N + c) * kMaxDeg + rank] = x;
+        if (x.y != 0.0) *b.cplx = 1;
       }
     }
     for (int i = lane; i < nn1; i += 32) {
@@ -382,32 +389,22 @@ __global__ void __launch_bounds__(128) k_bulk_vertex(BasisView B, int nP, const 
   }
 }
 
-// npd[p N + k]: nonzero components of D_1 .. D_k of channel p (p = nP: of h).
-__global__ void k_bulk_dcount(BasisView B, int nP, const double2* dl, const int* hasD, const double* h, int* npd) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x, N = B.N;
-  if (p > nP) return;
-  int n = 0;
-  npd[(int64_t)p * N] = 0;
-  for (int k = 1; k < N; ++k) {
-    bool nzc;
-    if (p == nP) {
-      nzc = h && h[2 * B.P - 1 + k] != 0.0;
-    } else {
-      const double2 x = hasD[p] ? dl[(int64_t)p * N + k] : make_double2(0.0, 0.0);
-      nzc = x.x != 0.0 || x.y != 0.0;
-    }
-    n += nzc;
-    npd[(int64_t)p * N + k] = n;
-  }
-}
-
 // exponent of |x|, 0 for zero
 __device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// |x| bit for bit: orders as the value does, NaN above all; -x.  Integer work: a warp instruction of the FP64 pipe
+// takes some 60 cycles whatever it computes.
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ double minus(double x, bool neg) {
+  return __longlong_as_double(__double_as_longlong(x) ^ (neg ? (long long)0x8000000000000000ull : 0ll));
+}
 
 // The rows of pair (c, d) by GW lanes, candidate e = i deg(d) + j: a = ucol[c][i],
 // b = ucol[d][j].  FILL = false: rowc of both rows, slow[row] = 1 for the rows of
 // the general way, the number of join terms of the others; FILL = true: the
-// entries at rowptr.
+// entries at rowptr.  Real l_p (the usual ladder) take two products of a term's
+// six; comparisons and signs are integer work.
 template <bool FILL, int GW>
 __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk b, unsigned long long* rowc,
                                                    unsigned long long* terms, const int64_t* rowptr, int32_t* col,
@@ -416,7 +413,8 @@ __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk 
   const unsigned gmask = (GW == 32 ? 0xffffffffu : ((1u << GW) - 1u)) << g0;
   // candidate counts of at most 4 x 4 take 16 lanes a pair
   if ((*b.maxdeg <= 4) != (GW == 16)) return;
-  const double lim = 1e-12 * *b.smax;
+  const unsigned long long lim = mag_bits(1e-12 * *b.smax);
+  const bool cplx = *b.cplx != 0;
   unsigned long long nterm = 0;
   for (int64_t w0 = (blockIdx.x * (int64_t)256 + (threadIdx.x & ~31)) / GW; w0 < B.P;
        w0 += gridDim.x * (int64_t)256 / GW) {
@@ -440,32 +438,39 @@ __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk 
     int mr = 0, mi = 0;  // largest exponent of the terms
     for (int p = 0; p < nP; ++p) {
       const double2 x = b.Lu[((int64_t)p * N + c) * kMaxDeg + i], y = b.Lu[((int64_t)p * N + d) * kMaxDeg + j];
-      const double gp = b.gamma[p];
-      const double gx = gp * x.x, gy = gp * x.y;
-      const double t0 = gx * y.x, t1 = gy * y.y, t2 = gy * y.x, t3 = gx * y.y;
-      mr = max(mr, max(expo(t0), expo(t1)));
+      // explicit rounding: the count and the fill have to see the same bits
+      const double gx = __dmul_rn(b.gamma[p], x.x), t0 = __dmul_rn(gx, y.x);
+      mr = max(mr, expo(t0));
+      if (!cplx) {
+        re = p ? __dadd_rn(re, t0) : t0;
+        continue;
+      }
+      const double gy = __dmul_rn(b.gamma[p], x.y);
+      const double t1 = __dmul_rn(gy, y.y), t2 = __dmul_rn(gy, y.x), t3 = __dmul_rn(gx, y.y);
+      mr = max(mr, expo(t1));
       mi = max(mi, max(expo(t2), expo(t3)));
-      re += t0 + t1;
-      im += t2 - t3;
+      re = __dadd_rn(re, __dadd_rn(t0, t1));
+      im = __dadd_rn(im, __dadd_rn(t2, -t3));
     }
     if (bc == d) {
       const double2 x = b.G[c * kMaxDeg + i];
       mr = max(mr, expo(x.x));
       mi = max(mi, expo(x.y));
-      re += x.x;
-      im += x.y;
+      re = __dadd_rn(re, x.x);
+      im = __dadd_rn(im, x.y);
     }
     if (ac == c) {
       const double2 x = b.G[d * kMaxDeg + j];
       mr = max(mr, expo(x.x));
       mi = max(mi, expo(x.y));
-      re += x.x;
-      im -= x.y;
+      re = __dadd_rn(re, x.x);
+      im = __dadd_rn(im, -x.y);
     }
     // zero up to the rounding of the terms; kept; or not certain
-    kre = expo(re) + 49 > mr && re != 0.0;
-    kim = expo(im) + 49 > mi && im != 0.0;
-    unsure = (kre && !(fabs(re) > lim)) || (kim && !(fabs(im) > lim));
+    const unsigned long long ur = mag_bits(re), ui = mag_bits(im), inf = 0x7ff0000000000000ull;
+    kre = expo(re) + 49 > mr && ur != 0;
+    kim = expo(im) + 49 > mi && ui != 0;
+    unsure = (kre && (ur <= lim || ur > inf)) || (kim && (ui <= lim || ui > inf));
     flip = ac > bc;
     pi = (int32_t)pair_index_any(N, ac, bc);
   }
@@ -525,13 +530,13 @@ __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk 
     col[rs + rr] = pi;
     val[rs + rr] = re;
     col[rj + nim + rr] = P + pi;
-    val[rj + nim + rr] = flip ? -re : re;
+    val[rj + nim + rr] = minus(re, flip);
   }
   if (kim) {  // A(S, J) and A(J, S)
     col[rs + nre + ri] = P + pi;
-    val[rs + nre + ri] = flip ? -im : im;
+    val[rs + nre + ri] = minus(im, flip);
     col[rj + ri] = pi;
-    val[rj + ri] = -im;
+    val[rj + ri] = minus(im, true);
   }
   }
   if (!FILL) {
@@ -567,7 +572,7 @@ size_t csr_bulk_bytes(int N, int nP) {
   auto r = [&](size_t x) { return (x + a - 1) & ~(a - 1); };
   return r(16 * nn * nP) + r(8 * nn * nP) + r(4 * nn) + r(nn) + r(8 * (size_t)N) + r(4 * (size_t)N * kMaxDeg) +
          r(16 * (size_t)N * kMaxDeg) + r(16 * (size_t)N * kMaxDeg * nP) + 2 * r(4 * (size_t)N * kMaxNear) +
-         4 * r(4 * (size_t)N) + r(4 * (size_t)N * (nP + 1)) + 4 * a + r(nn) + 2 * r(8 * (size_t)(nP + 1));
+         4 * r(4 * (size_t)N) + r(4 * (size_t)N * (nP + 1)) + 5 * a + r(nn) + 2 * r(8 * (size_t)(nP + 1));
 }
 
 CsrBulk csr_bulk_carve(void* mem, int N, int nP, const double* gamma) {
@@ -579,13 +584,14 @@ CsrBulk csr_bulk_carve(void* mem, int N, int nP, const double* gamma) {
   };
   const size_t nn = (size_t)N * N;
   CsrBulk b{};
-  // zeroed by csr_bulk_count: L, mag, cnt, near, smax, maxdeg, mx, gd
+  // zeroed by csr_bulk_count: L, mag, cnt, near, smax, maxdeg, cplx, mx, gd
   b.L = static_cast<double2*>(take(16 * nn * nP));
   b.mag = static_cast<double*>(take(8 * nn * nP));
   b.cnt = static_cast<int*>(take(4 * nn));
   b.near = static_cast<uint8_t*>(take(nn));
   b.smax = static_cast<double*>(take(8));
   b.maxdeg = static_cast<int*>(take(4));
+  b.cplx = static_cast<int*>(take(4));
   b.mx = static_cast<double*>(take(8 * (size_t)(nP + 1)));
   b.gd = static_cast<double*>(take(8 * (size_t)(nP + 1)));
   b.zeroed = (size_t)(p - static_cast<char*>(mem));
@@ -620,15 +626,14 @@ cudaError_t csr_bulk_count(const lb::BasisView& B, const CsrBulk& b, int nP, con
     k_bulk_clean<<<nb(nn, 256), 256, 0, st>>>(nn, b.L, b.mag);
     note_launch(2);
   }
-  k_bulk_diag<<<nP + 1, 256, 0, st>>>(B, nP, dl, hasD, h, b);
+  k_bulk_diag<<<nP + 1, kSuffixThreads, 0, st>>>(B, nP, dl, hasD, h, b);
   k_bulk_vertex<<<nb(N, 4), 128, 0, st>>>(B, nP, h, b.gamma, b);
   k_bulk_limit<<<1, 1, 0, st>>>(nP, b);
-  k_bulk_dcount<<<nb(nP + 1, 32), 32, 0, st>>>(B, nP, dl, hasD, h, b.npd);
   const unsigned grid = (unsigned)std::min<int64_t>(nb(B.P * 16, 256), 152 * 16);
   k_bulk_rows<false, 16><<<grid, 256, 0, st>>>(B, nP, b, rowc, terms, nullptr, nullptr, nullptr);
   k_bulk_rows<false, 32><<<grid, 256, 0, st>>>(B, nP, b, rowc, terms, nullptr, nullptr, nullptr);
   k_bulk_list<<<nb(B.M, 256), 256, 0, st>>>(B.M, 2 * B.P, b.slow, list, nlist);
-  note_launch(7);
+  note_launch(6);
   return cudaGetLastError();
 }
 

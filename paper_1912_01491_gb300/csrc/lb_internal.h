@@ -87,7 +87,7 @@ struct CsrBulk {
   int* cnt;             // N x N: list entries on the edge
   uint8_t* near;        // N x N: 1: the rows of this pair go the general way
   double *smax, *mx, *gd;
-  int* maxdeg;
+  int *maxdeg, *cplx;   // most candidates of a vertex; 1: an element of an L_p at them has an imaginary part
   double* hdiag;        // N
   int* ucol;            // candidates of a vertex, and G, L_p at them
   double2 *G, *Lu;

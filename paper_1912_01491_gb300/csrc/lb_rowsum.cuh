@@ -90,4 +90,26 @@ __device__ __forceinline__ double lane_sum(const float (&a)[4]) {
   return lane_sum_tree(a);
 }
 
+// The sum of x over the threads of the block behind the calling one (blocks of
+// kSuffixThreads, sh: one value per warp).
+constexpr int kSuffixThreads = 256;
+
+template <class T>
+__device__ __forceinline__ T block_suffix(T x, T* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  T in = x;  // inclusive
+  for (int o = 1; o < 32; o <<= 1) {
+    const T u = __shfl_down_sync(0xffffffffu, in, o);
+    if (lane + o < 32) in += u;
+  }
+  T ex = __shfl_down_sync(0xffffffffu, in, 1);
+  if (lane == 31) ex = T(0);
+  __syncthreads();
+  if (lane == 0) sh[wid] = in;
+  __syncthreads();
+  T behind = T(0);
+  for (int w = kSuffixThreads / 32 - 1; w > wid; --w) behind += sh[w];
+  return ex + behind;
+}
+
 }  // namespace lb

@@ -59,7 +59,7 @@ def _ops(model, N):
     return H, [(g, L)]
 
 
-@pytest.mark.parametrize("N", [64, 77])
+@pytest.mark.parametrize("N", [64, 131])
 @pytest.mark.parametrize("model", ["ladder", "dimer", "complex", "two steps", "graph", "no H", "weak channel",
                                    "weak edges", "negative", "hub"])
 def test_closed_rows_equal_oracle_and_join(model, N):
@@ -89,11 +89,11 @@ def test_closed_rows_equal_oracle_and_join(model, N):
         b.close()
 
 
-def test_join_terms_and_repeated_entries():
+@pytest.mark.parametrize("N", [70, 130])
+def test_join_terms_and_repeated_entries(N):
     """The number of join terms does not depend on which rows are closed, and
     an index listed twice counts twice."""
     import paper_1912_01491_gb300 as lb
-    N = 70
     with lb.Basis(N) as B:
         for model in ("ladder", "dimer", "graph"):
             H, [(g, L)] = _ops(model, N)
