@@ -949,7 +949,9 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
     cudaMemPool_t p = nullptr;
     if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
     uint64_t keep = kScratchKeep;
-    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+    int off = 0;  // no waiting of one stream for another's memory
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess ||
+        (e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &off)) != cudaSuccess) {
       cudaMemPoolDestroy(p);
       return e;
     }

@@ -186,6 +186,7 @@ struct BatchItem {
   double* v;          // M, in/out
 };
 constexpr int kBatchMaxN = 64;
+constexpr int kBatchSide = 5;  // side streams of a batch: one per cluster size
 
 // propagator form (lb_prop.cu): batched Y = B + alpha A G over square
 // M x M row-major matrices (B may be null), one launch over the 64 x 64
