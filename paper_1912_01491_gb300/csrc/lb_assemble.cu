@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(256) k_assemble(BasisView B, AView A, const do
 
 // Eq. (08): k_s = (i/N) sum_jk a_jk f_jks = -(1/N) sum_jk Im(a_jk) f_jks.
 // One warp per s; lanes stride over the j candidates.
-// CLOSED: the diagonal rows are left to k_kvec_diag_* below.
+// CLOSED: the diagonal rows are left to kvec_diag below.
 template <bool CLOSED>
 __global__ void k_kvec(BasisView B, AView A, double* __restrict__ K) {
   const int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -427,11 +427,11 @@ __global__ void k_kvec(BasisView B, AView A, double* __restrict__ K) {
 //   K_{D_nu} = -(1/N) sum_{x<y} (delta_x(nu) - delta_y(nu)) g_xy
 //            = -(1/N) sum_k delta_k(nu) G_k,  G_k = sum_{y>k} g_ky - sum_{x<k} g_xk,
 // and sum_k delta_k(nu) G_k = c_nu sum_{k<nu} G_k - nu c_nu G_nu (the prefix
-// form of the Helmert vectors).  k_kvec_diag_g: one block per vertex k, a
-// fixed-order reduction; k_kvec_diag: the prefix over k (one warp) and the
-// rows.
-__global__ void __launch_bounds__(128) k_kvec_diag_g(BasisView B, AView A, double* __restrict__ G) {
-  const int N = B.N, k = blockIdx.x;
+// form of the Helmert vectors).  kvec_vertex: G_k by one block of 128, in a
+// fixed order; kvec_diag: the prefix over k (one warp) and the rows, by one
+// block, pre holding N + 1 values.
+__device__ __forceinline__ void kvec_vertex(const BasisView& B, const AView& A, int k, double* G) {
+  const int N = B.N;
   double acc = 0.0;
   for (int u = threadIdx.x; u < N; u += blockDim.x) {
     if (u == k) continue;
@@ -449,14 +449,12 @@ __global__ void __launch_bounds__(128) k_kvec_diag_g(BasisView B, AView A, doubl
 __device__ __forceinline__ void warp_prefix(double* arr, int n);  // below
 __device__ __forceinline__ void warp_suffix(const double* x, double* y, int n);  // below
 
-__global__ void __launch_bounds__(256) k_kvec_diag(BasisView B, const double* __restrict__ G,
-                                                    double* __restrict__ K) {
-  __shared__ double pre[lbi::kMaxDenseN + 1];  // pre[nu] = sum_{k < nu} G_k
+__device__ __forceinline__ void kvec_diag(const BasisView& B, const double* G, double* K, double* pre) {
   const int N = B.N;
   for (int k = threadIdx.x; k < N; k += blockDim.x) pre[k + 1] = G[k];
   if (threadIdx.x == 0) pre[0] = 0.0;
   __syncthreads();
-  if (threadIdx.x < 32) warp_prefix(pre, N);
+  if (threadIdx.x < 32) warp_prefix(pre, N);  // pre[nu] = sum_{k < nu} G_k
   __syncthreads();
   for (int nu = 1 + threadIdx.x; nu < N; nu += blockDim.x)
     K[d_index(B, nu)] = -(ld_c(B, nu) * pre[nu] + ld_lc(B, nu) * G[nu]) / (double)N;
@@ -1014,11 +1012,11 @@ __device__ __forceinline__ bool quad_tile_seek(int N, int q, QuadTile& T, int64_
   return true;
 }
 
-constexpr int kQuadThreads = 256;
 // at most 168 registers: no spills, and a little faster than the 182 the
 // compiler takes without a cap
 __global__ void __maxnreg__(168) k_disjoint4(BasisView B, AView A, double* __restrict__ Aout,
                                                                double* __restrict__ Qout, double* __restrict__ Rout) {
+  grid_release();
   const int N = B.N;
   const int64_t P = B.P, M = B.M;
   const int64_t pq = blockIdx.x;
@@ -1068,6 +1066,7 @@ __global__ void __maxnreg__(168) k_disjoint4(BasisView B, AView A, double* __res
     I = In;
     cur = nxt;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) grid_wait();  // complete behind the grids before this one
 }
 
 // Pair row s = (as, bs) type ts, diagonal columns n = D_nu.  One block per
@@ -1337,54 +1336,49 @@ struct DDTables {
   }
 };
 
-// Row x of W and V, and their row suffixes.  One block per x.
-__global__ void __launch_bounds__(128) k_dd_rows(BasisView B, AView A, DDTables T) {
-  const int N = B.N, x = blockIdx.x;
+// Row x of W and V, and their row suffixes (one block; sh: 4 (N + 1) values).
+__device__ __forceinline__ void dd_row(const BasisView& B, const AView& A, const DDTables& T, int x, double* sh) {
+  const int N = B.N, L = N + 1;
   for (int y = threadIdx.x; y < N; y += blockDim.x) {
     double W = 0.0, V = 0.0;
     if (y > x) dd_wv(B, A, x, y, W, V);
-    T.W[(int64_t)x * N + y] = W;
-    T.V[(int64_t)x * N + y] = V;
+    T.W[(int64_t)x * N + y] = sh[y] = W;
+    T.V[(int64_t)x * N + y] = sh[L + y] = V;
   }
   __syncthreads();
-  if (threadIdx.x < 2) {
-    const double* X = (threadIdx.x ? T.V : T.W) + (int64_t)x * N;
-    double* RS = (threadIdx.x ? T.RSV : T.RSW) + (int64_t)x * (N + 1);
-    double acc = 0.0;
-    RS[N] = 0.0;
-    for (int b = N - 1; b >= 0; --b) {
-      if (b > x) acc += X[b];
-      RS[b] = acc;
-    }
+  const int wid = threadIdx.x >> 5;
+  if (wid < 2) warp_suffix(sh + wid * L, sh + (2 + wid) * L, N);
+  __syncthreads();
+  for (int b = threadIdx.x; b <= N; b += blockDim.x) {
+    T.RSW[(int64_t)x * L + b] = sh[2 * L + b];
+    T.RSV[(int64_t)x * L + b] = sh[3 * L + b];
   }
 }
 
-// Column prefixes CP[y][a] and corner sums C[a][b] = sum_{x<a} RS[x][b]:
-// thread t < 2N takes column y = t / 2 (W or V), thread t in [2N, 4N + 2)
-// takes corner column b.
-__global__ void __launch_bounds__(128) k_dd_cols(BasisView B, DDTables T) {
-  const int N = B.N;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < 2 * N) {
-    const int y = t >> 1, wv = t & 1;
-    const double* X = wv ? T.V : T.W;
-    double* CP = (wv ? T.CPV : T.CPW) + (int64_t)y * (N + 1);
-    double acc = 0.0;
-    CP[0] = 0.0;
-    for (int a = 0; a < N; ++a) {
-      if (a < y) acc += X[(int64_t)a * N + y];
-      CP[a + 1] = acc;
+// Column prefixes CP[y][a] and corner sums C[a][b] = sum_{x<a} RS[x][b]: one
+// warp per column, u < 2N: column y = u / 2 of W or V, u in [2N, 4N + 2):
+// corner column b; 32 rows at a time.
+__device__ __forceinline__ void dd_col(const BasisView& B, const DDTables& T, int u) {
+  const int N = B.N, lane = threadIdx.x & 31;
+  const bool corner = u >= 2 * N;
+  const int y = (corner ? u - 2 * N : u) >> 1, wv = u & 1;
+  const int64_t from = corner ? N + 1 : N;                   // row stride of the terms
+  const double* X = (corner ? (wv ? T.RSV : T.RSW) : (wv ? T.V : T.W)) + y;
+  const int64_t to = corner ? N + 1 : 1;                     // stride of the sums
+  double* S = corner ? (wv ? T.CV : T.CW) + y : (wv ? T.CPV : T.CPW) + (int64_t)y * (N + 1);
+  double carry = 0.0;
+  if (lane == 0) S[0] = 0.0;
+  for (int a0 = 0; a0 < N; a0 += 32) {
+    const int a = a0 + lane;
+    double t = a < N ? X[a * from] : 0.0;  // W and V are zero for a >= y
+    if (lane == 0) t += carry;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double up = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += up;
     }
-  } else if (t < 2 * N + 2 * (N + 1)) {
-    const int u = t - 2 * N, b = u >> 1, wv = u & 1;
-    const double* RS = wv ? T.RSV : T.RSW;
-    double* C = wv ? T.CV : T.CW;
-    double acc = 0.0;
-    C[b] = 0.0;  // a = 0
-    for (int a = 1; a <= N; ++a) {
-      acc += RS[(int64_t)(a - 1) * (N + 1) + b];
-      C[(int64_t)a * (N + 1) + b] = acc;
-    }
+    if (a < N) S[(a + 1) * to] = t;
+    carry = __shfl_sync(0xffffffffu, t, 31);
   }
 }
 
@@ -1397,45 +1391,40 @@ __device__ __forceinline__ double dd_cell(const double* X, const double* RS, con
   return C[(int64_t)x1 * (N + 1) + y0] - C[(int64_t)x1 * (N + 1) + y1];  // x0 = 0
 }
 
-// One thread per entry (nu, mu), nu, mu in 1..N-1.
-__global__ void __launch_bounds__(256) k_dd_cells(BasisView B, DDTables T, double* __restrict__ Aout,
+// 16 lanes per entry (nu, mu), nu, mu in 1..N-1, one for each of the ten cells:
+// the cells of an entry in turn are a chain of some hundred FP64 instructions
+// and loads (one thread an entry: 16 us at N = 10 and 50 alike, now 5).
+constexpr int kCellThreads = 64;
+__global__ void __launch_bounds__(kCellThreads) k_dd_cells(BasisView B, DDTables T, double* __restrict__ Aout,
                                                   double* __restrict__ Qout, double* __restrict__ Rout) {
+  grid_release();
+  grid_wait();
   const int N = B.N;
   const int64_t M = B.M;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)(N - 1) * (N - 1)) return;
-  const int nu = 1 + (int)(e / (N - 1)), mu = 1 + (int)(e % (N - 1));
+  const int64_t e = ((int64_t)blockIdx.x * kCellThreads + threadIdx.x) >> 4;
+  const int t = threadIdx.x & 15;
+  const bool in = e < (int64_t)(N - 1) * (N - 1);
+  const int nu = in ? 1 + (int)(e / (N - 1)) : 1, mu = in ? 1 + (int)(e % (N - 1)) : 1;
   const int lo = imin(nu, mu), hi = imax(nu, mu);
-  int c0[5], c1[5], nc = 0;
-  auto add = [&](int a, int b) {
-    if (b > a) {
-      c0[nc] = a;
-      c1[nc] = b;
-      ++nc;
-    }
-  };
-  add(0, lo);
-  add(lo, lo + 1);
-  if (hi > lo) {
-    add(lo + 1, hi);
-    add(hi, hi + 1);
-  }
-  add(hi + 1, N);
-  double acc = 0.0;
-  for (int i = 0; i < nc; ++i) {
-    const int x = c0[i];
-    const double dxn = dlt(B, x, nu), dxm = dlt(B, x, mu);
-    for (int j = i + 1; j < nc; ++j) {
-      const int y = c0[j];
-      const double g = dxn - dlt(B, y, nu);
-      if (g == 0.0) continue;
-      const double dym = dlt(B, y, mu);
+  double term = 0.0;
+  if (in && t < 10) {
+    // t = (0, 1), (0, 2), .. (3, 4)
+    const int i = t < 4 ? 0 : t < 7 ? 1 : t < 9 ? 2 : 3, j = t < 4 ? t + 1 : t < 7 ? t - 2 : t < 9 ? t - 4 : 4;
+    auto begin = [&](int k) { return k == 0 ? 0 : k == 1 ? lo : k == 2 ? lo + 1 : k == 3 ? hi : hi + 1; };
+    auto end = [&](int k) { return k == 0 ? lo : k == 1 ? lo + 1 : k == 2 ? hi : k == 3 ? (hi > lo ? hi + 1 : hi) : N; };
+    const int x0 = begin(i), x1 = end(i), y0 = begin(j), y1 = end(j);
+    if (x1 > x0 && y1 > y0) {
+      const double dxn = dlt(B, x0, nu), dxm = dlt(B, x0, mu);
+      const double g = dxn - dlt(B, y0, nu);
+      const double dym = dlt(B, y0, mu);
       const double cw = g * (dxm - dym), cv = 2.0 * g * (dxm + dym);
-      if (cw != 0.0) acc = fma(cw, dd_cell(T.W, T.RSW, T.CPW, T.CW, N, c0[i], c1[i], c0[j], c1[j]), acc);
-      if (cv != 0.0) acc = fma(cv, dd_cell(T.V, T.RSV, T.CPV, T.CV, N, c0[i], c1[i], c0[j], c1[j]), acc);
+      if (cw != 0.0) term = cw * dd_cell(T.W, T.RSW, T.CPW, T.CW, N, x0, x1, y0, y1);
+      if (cv != 0.0) term = fma(cv, dd_cell(T.V, T.RSV, T.CPV, T.CV, N, x0, x1, y0, y1), term);
     }
   }
-  const double r = -0.5 * acc;
+  for (int o = 8; o > 0; o >>= 1) term += __shfl_xor_sync(0xffffffffu, term, o);
+  if (!in || t != 0) return;
+  const double r = -0.5 * term;
   const int64_t o = d_index(B, nu) * M + d_index(B, mu);
   if (Rout) Rout[o] = r;
   if (Qout) Qout[o] = 0.0;
@@ -1445,12 +1434,12 @@ __global__ void __launch_bounds__(256) k_dd_cells(BasisView B, DDTables T, doubl
 // Tables of the D x D block X[lam][mu] = a[D_lam][D_mu] for the same-edge
 // entries' D-section sums: CXr[lam][mu] = c_lam Re X[lam][mu] and the
 // suffix sums SXi[k][mu] = sum_{lam >= k} c_lam Im X[lam][mu] (k = 0..N,
-// SXi[N][mu] = 0).  One block per column mu >= 1; row-major N-wide tables.
-__global__ void __launch_bounds__(128) k_dtab(BasisView B, AView A, double* __restrict__ CXr,
-                                              double* __restrict__ SXi) {
-  __shared__ double xi[lbi::kMaxDenseN];
-  __shared__ double sx[lbi::kMaxDenseN + 1];
-  const int N = B.N, mu = 1 + blockIdx.x;
+// SXi[N][mu] = 0).  One block per column mu >= 1; row-major N-wide tables; sh:
+// 2 (N + 1) values.
+__device__ __forceinline__ void dtab_col(const BasisView& B, const AView& A, int mu, double* CXr, double* SXi,
+                                         double* sh) {
+  const int N = B.N;
+  double *xi = sh, *sx = sh + N + 1;
   for (int lam = threadIdx.x; lam < N; lam += blockDim.x) {
     double cr = 0.0, ci = 0.0;
     if (lam >= 1) {
@@ -1466,6 +1455,18 @@ __global__ void __launch_bounds__(128) k_dtab(BasisView B, AView A, double* __re
   if (threadIdx.x < 32) warp_suffix(xi, sx, N);
   __syncthreads();
   for (int k = threadIdx.x; k <= N; k += blockDim.x) SXi[(int64_t)k * N + mu] = sx[k];
+}
+
+// The tables the closed form needs first, a block each: nd rows of W and V, nk
+// vertex sums of K's diagonal rows, the columns of the D x D tables.
+__global__ void __launch_bounds__(128) k_tables(BasisView B, AView A, DDTables T, double* __restrict__ G,
+                                                double* __restrict__ CXr, double* __restrict__ SXi, int nd, int nk) {
+  extern __shared__ double st_sh[];  // 4 (N + 1)
+  const int i = blockIdx.x;
+  grid_release();
+  if (i < nd) dd_row(B, A, T, i, st_sh);
+  else if (i < nd + nk) kvec_vertex(B, A, i - nd, G);
+  else dtab_col(B, A, 1 + i - nd - nk, CXr, SXi, st_sh);
 }
 
 // Pair-pair entries whose edges share one vertex v: s on (v, p), n on (v, q).
@@ -1873,6 +1874,7 @@ __global__ void __launch_bounds__(256, 3) k_shared_closed(BasisView B, AView A, 
                                                        double* __restrict__ Aout, double* __restrict__ Qout,
                                                        double* __restrict__ Rout) {
   extern __shared__ double sc[];
+  grid_release();
   const int N = B.N;
   const int64_t P = B.P, M = B.M;
   const int32_t ab = __ldg(B.pair_ab + blockIdx.x);
@@ -1908,11 +1910,11 @@ __global__ void __launch_bounds__(256, 3) k_shared_closed(BasisView B, AView A, 
   }
   __syncthreads();
   {
-    // warps 0..3: suffix sums of CX[0], CX[1], CY[0], CY[1] into the (not
+    // suffix sums of CX[0], CX[1], CY[0], CY[1] into the (not
     // yet used) SU arrays: sums of the terms mu > k only, never a total
     // minus the terms below k
-    const int wi = threadIdx.x >> 5;
-    if (wi < 4) warp_suffix(wi < 2 ? CX + wi * L : CY + (wi - 2) * L, SU + wi * L, N);
+    for (int wi = threadIdx.x >> 5; wi < 4; wi += blockDim.x >> 5)
+      warp_suffix(wi < 2 ? CX + wi * L : CY + (wi - 2) * L, SU + wi * L, N);
   }
   __syncthreads();
   // (D x)_k for the four staged D-column vectors: sum_{mu > k} c_mu x_mu + delta_k(k) x_k
@@ -1930,8 +1932,8 @@ __global__ void __launch_bounds__(256, 3) k_shared_closed(BasisView B, AView A, 
   // total is a signed sum of three range sums of one staged array: 8 arrays
   // (PX and PY of the four (tj, tk)) x 3 ranges, 8 threads per range sum.
   __shared__ double RS[8][3];
-  if (threadIdx.x < 24 * 8) {
-    const int c = threadIdx.x >> 3, sub = threadIdx.x & 7;
+  for (int c = threadIdx.x >> 3; c < 24; c += blockDim.x >> 3) {  // whole warps: 24 and blockDim / 8 are multiples of 4
+    const int sub = threadIdx.x & 7;
     const int arr = c / 3, rg = c % 3;
     const double* X = (arr < 4 ? PX : PY) + (arr & 3) * L;
     const int lo = rg == 0 ? 0 : (rg == 1 ? p + 1 : q + 1), hi = rg == 0 ? p : (rg == 1 ? q : N);
@@ -1988,11 +1990,12 @@ __global__ void __launch_bounds__(256, 3) k_shared_closed(BasisView B, AView A, 
   if (threadIdx.x < 4) PU[threadIdx.x * L] = 0.0;
   __syncthreads();
   {
-    const int wi = threadIdx.x >> 5;  // warps 0..3: prefix of U, 4..7: suffix
-    if (wi < 4)
-      warp_prefix(PU + wi * L, N);
-    else if (wi < 8)
-      warp_suffix(RU + (wi - 4) * L, SU + (wi - 4) * L, N);
+    for (int wi = threadIdx.x >> 5; wi < 8; wi += blockDim.x >> 5) {  // 0..3: prefix of U, 4..7: suffix
+      if (wi < 4)
+        warp_prefix(PU + wi * L, N);
+      else
+        warp_suffix(RU + (wi - 4) * L, SU + (wi - 4) * L, N);
+    }
   }
   __syncthreads();
   // pair x pair, edges sharing a vertex: 2 orientations x N vertices v, the
@@ -2055,6 +2058,7 @@ __global__ void __launch_bounds__(256, 3) k_shared_closed(BasisView B, AView A, 
     if (Qout) Qout[o] = qv;
     if (Aout) Aout[o] = qv + r;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) grid_wait();  // complete behind the grids before this one
 }
 
 // Closed-form k_pd (pair row s, diagonal columns D_nu) and, when K is
@@ -2081,6 +2085,7 @@ __global__ void __launch_bounds__(kRowThreads) k_pd_closed(BasisView B, AView A,
                                                            double* __restrict__ Aout, double* __restrict__ Qout,
                                                            double* __restrict__ Rout, double* __restrict__ K) {
   extern __shared__ double sq[];
+  grid_release();
   const int N = B.N;
   const int64_t P = B.P, M = B.M;
   const int64_t s = blockIdx.x;
@@ -2218,6 +2223,7 @@ __global__ void __launch_bounds__(kRowThreads) k_pd_closed(BasisView B, AView A,
     if (Qout) Qout[o] = q;
     if (Aout) Aout[o] = q + r;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) grid_wait();  // complete behind the grids before this one
 }
 
 // Pair-pair entries on the same edge (a, b): s, n in {S_ab, J_ab}.  One block
@@ -2310,14 +2316,25 @@ __global__ void __launch_bounds__(kSameThreads) k_same(BasisView B, AView A, dou
 // a[(tj, (v', w))][(tk, (v', w))], tj, tk in {S, J}, are loaded once and
 // enter every (ts, tn, tl) term (the per-pair sums keep the order of one pair
 // at a time); the l = partner(s) part sums the D x D block over the edge's
-// window from the tables of k_dtab.  The block also forms the entries'
+// window from the D x D tables.  The block also forms the entries'
 // D-section part (by completeness, -+Re a of the partner pair) and Q, and
-// writes the four entries whole.
+// writes the four entries whole.  The blocks past the ns edges take the second
+// half of the tables: a warp per column prefix and corner sum (nc of them), and
+// the last block, if K is given, K's diagonal rows.
 __global__ void __launch_bounds__(kSameThreads) k_same_closed(BasisView B, AView A, const double* __restrict__ h,
-                                                              const double* __restrict__ CXr,
-                                                              const double* __restrict__ SXi,
+                                                              const double* CXr, const double* SXi,
                                                               double* __restrict__ Aout, double* __restrict__ Qout,
-                                                              double* __restrict__ Rout) {
+                                                              double* __restrict__ Rout, int ns, int nc, DDTables T,
+                                                              const double* G, double* __restrict__ K) {
+  grid_release();
+  if ((int)blockIdx.x >= ns) {
+    __shared__ double pre[lbi::kMaxDenseN + 1];
+    grid_wait();
+    const int u = ((int)blockIdx.x - ns) * (kSameThreads / 32) + (threadIdx.x >> 5);
+    if (K != nullptr && blockIdx.x == gridDim.x - 1) kvec_diag(B, G, K, pre);
+    else if (u < nc) dd_col(B, T, u);
+    return;
+  }
   __shared__ double red[5][kSameThreads];  // per thread: the four entries' sums, the Q sum
   __shared__ double tot[5];
   const int N = B.N;
@@ -2363,6 +2380,7 @@ __global__ void __launch_bounds__(kSameThreads) k_same_closed(BasisView B, AView
   // f sum term by term over the window (a difference of two longer sums
   // would cancel terms outside it, with their rounding).
   double tf = 0.0, td = 0.0;
+  grid_wait();  // the tables
   {
     const int lo = imax(a, 1);
     for (int mu = lo + threadIdx.x; mu <= b; mu += blockDim.x) {
@@ -2524,6 +2542,133 @@ cudaError_t upload_hermitian(const double2* host, double2* dev, int64_t M, cudaS
   return cudaGetLastError();
 }
 
+// Launch behind what is queued on st; overlap: the grids before it may still
+// run (they have all released it, and it waits where it reads what they write).
+template <class... P, class... X>
+static cudaError_t launch_on(bool overlap, void (*kernel)(P...), int64_t grid, int threads, size_t smem,
+                             cudaStream_t st, X... x) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  note_launch(1);
+  return cudaLaunchKernelEx(&cfg, kernel, P(x)...);
+}
+
+// Threads of a block.  k_disjoint4 (168 registers): blocks of 128 put 12 warps
+// on an SM, of 256 only 8, but the warps of a large block walk neighbouring
+// output sectors together, which decides where the matrix exceeds L2 (the whole
+// assembly with 128 / 256: N = 30 45 / 47 us, N = 50 136 / 157, N = 100 1180 /
+// 1198, N = 140 4.2 / 3.7 ms, N = 200 18.1 / 13.2 ms).  k_shared_closed: its
+// loops run over 2N items, so up to N = 64 blocks of 128 lose nothing and twice
+// as many fit an SM; with fewer than a wave of blocks (3 of 256 an SM) the
+// larger ones are quicker (128 / 256: N = 10 21.4 / 20.4 us, N = 30 41.1 / 44.7,
+// N = 50 131 / 136, N = 80 equal, N = 140 4.6 / 3.7 ms).
+static int quad_threads(int N) { return N <= 100 ? 128 : 256; }
+static int shared_threads(int N, int64_t blocks) { return N <= 64 && blocks > 3 * 152 ? 128 : 256; }
+
+// The closed algorithm.  Its six kernels write disjoint entries; only the
+// same-edge kernel needs tables of k_tables and k_dd_cells those of both.  At
+// small N each is a chain of a few microseconds on part of the chip (N = 10:
+// 3 to 17 us each, 77 us in a row; now 20 us in all), so they are launched to
+// overlap, the dependent ones first (N = 50: 245 -> 131 us); at large N only the
+// tails do (N = 200: 13.4 -> 13.2 ms).
+static cudaError_t assemble_closed(const lb::BasisView& B, const double* h, const double2* a, double* A, double* Q,
+                                   double* R, double* K, cudaStream_t st, cudaEvent_t* ev) {
+  const AView av{a, B.M};
+  const int N = B.N;
+  const bool dense_out = A || Q || R, overlap = ev == nullptr;
+  if (!dense_out && !K) return cudaSuccess;
+  // scratch: the D x D tables, the vertex sums of K's diagonal rows, the diagonal x diagonal tables; from the
+  // retained pool: after a synchronization the default one would go to the driver again (0.15 ms)
+  const size_t g_at = 3 * (size_t)N * N, dd_at = g_at + N;
+  double* scratch = nullptr;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = scratch_pool(&pool);
+  if (e == cudaSuccess)
+    e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch),
+                                sizeof(double) * (dd_at + DDTables::doubles(N)), pool, st);
+  if (e != cudaSuccess) return e;
+  double *CXr = scratch, *SXi = scratch + (size_t)N * N, *G = scratch + g_at;  // N x N, (N + 1) x N, N
+  const DDTables T = DDTables::carve(scratch + dd_at, N);
+  const int nd = dense_out ? N : 0, nk = K ? N : 0;
+  auto tables = [&](bool ov) {
+    return launch_on(ov, k_tables, nd + nk + (dense_out ? N - 1 : 0), 128, sizeof(double) * 4 * (size_t)(N + 1), st, B,
+                     av, T, G, CXr, SXi, nd, nk);
+  };
+  auto same = [&](bool ov) {
+    const int ns = dense_out ? (int)B.P : 0, nc = dense_out ? 4 * N + 2 : 0, per = kSameThreads / 32;
+    return launch_on(ov, k_same_closed, ns + (nc + per - 1) / per + (K ? 1 : 0), kSameThreads, 0, st, B, av, h, CXr,
+                     SXi, A, Q, R, ns, nc, T, G, K);
+  };
+  auto cells = [&](bool ov) {
+    const int64_t n = 16 * (int64_t)(N - 1) * (N - 1);
+    return launch_on(ov, k_dd_cells, (n + kCellThreads - 1) / kCellThreads, kCellThreads, 0, st, B, T, A, Q, R);
+  };
+  auto shared = [&](bool ov) {
+    return launch_on(ov, k_shared_closed, B.P, shared_threads(N, B.P), sizeof(double) * 32 * (size_t)(N + 1), st, B, av, h, A, Q, R);
+  };
+  auto disjoint = [&](bool ov) {
+    return N < 4 ? cudaSuccess : launch_on(ov, k_disjoint4, B.P, quad_threads(N), 0, st, B, av, A, Q, R);
+  };
+  auto pair_diag = [&](bool ov) {
+    return launch_on(ov, k_pd_closed, 2 * B.P, kRowThreads, sizeof(double) * 6 * (size_t)(N + 1), st, B, av, h, A, Q,
+                     R, K);
+  };
+  auto run = [&](auto step, bool ov) {
+    if (e == cudaSuccess) e = step(ov);
+  };
+  if (overlap) {
+    if (!dense_out) {  // K alone: its pair rows too (else from k_pd_closed)
+      k_kvec<true><<<(unsigned)((2 * B.P * 32 + 255) / 256), 256, 0, st>>>(B, av, K);
+      note_launch(1);
+    }
+    run(tables, false);
+    run(same, true);
+    if (dense_out) {
+      run(cells, true);
+      run(shared, true);
+      run(disjoint, true);
+      run(pair_diag, true);
+    }
+  } else {
+    auto mark = [&](int i) {
+      if (e == cudaSuccess) e = cudaEventRecord(ev[i], st);
+    };
+    mark(0);
+    if (dense_out) run(disjoint, false);
+    mark(1);
+    if (dense_out) run(pair_diag, false);
+    mark(2);
+    mark(3);
+    run(tables, false);
+    mark(4);
+    if (dense_out) run(shared, false);
+    mark(5);
+    run(same, false);
+    if (dense_out) run(cells, false);
+    mark(6);
+    if (!dense_out) {
+      k_kvec<true><<<(unsigned)((2 * B.P * 32 + 255) / 256), 256, 0, st>>>(B, av, K);
+      note_launch(1);
+    }
+    mark(7);
+  }
+  const cudaError_t ef = cudaFreeAsync(scratch, st);
+  if (e == cudaSuccess) e = ef;
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double2* a, double* A,
                            double* Q, double* R, double* K, int algorithm, cudaStream_t st,
                            cudaEvent_t* ev) {
@@ -2532,7 +2677,7 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
   const int64_t P2 = 2 * B.P;
   const int64_t chunks = (P2 + 255) / 256;
   if (P2 * chunks > 0x7fffffffLL || N > kMaxDenseN) return cudaErrorInvalidConfiguration;
-  const bool closed = algorithm == LB_ALG_CLOSED;
+  if (algorithm == LB_ALG_CLOSED) return assemble_closed(B, h, a, A, Q, R, K, st, ev);
   cudaError_t e = cudaSuccess;
   // ev (optional, kAssembleKernels + 1 events): recorded before the first and
   // after every kernel of the sequence below, launched or not.
@@ -2541,126 +2686,53 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
   };
   mark(0);
   const bool dense_out = A || Q || R;
-  // 0: pair x pair (closed: disjoint edges, one lane per vertex quadruple in warp tiles)
+  // 0: pair x pair
   if (dense_out) {
-    if (closed) {
-      if (N >= 4) {
-        k_disjoint4<<<(unsigned)B.P, kQuadThreads, 0, st>>>(B, av, A, Q, R);
-        note_launch(1);
-      }
-    } else {
-      k_entries<LB_ALG_JOIN><<<(unsigned)(P2 * chunks), 256, 0, st>>>(B, av, h, A, Q, R);
-      note_launch(1);
-    }
+    k_entries<LB_ALG_JOIN><<<(unsigned)(P2 * chunks), 256, 0, st>>>(B, av, h, A, Q, R);
+    note_launch(1);
   }
   mark(1);
   // 1: pair x diagonal
   if (dense_out && e == cudaSuccess) {
-    if (closed) {
-      const size_t smem = sizeof(double) * 6 * (size_t)(N + 1);
-      e = cudaFuncSetAttribute(k_pd_closed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) k_pd_closed<<<(unsigned)P2, kRowThreads, smem, st>>>(B, av, h, A, Q, R, K);
-    } else {
-      const size_t smem = sizeof(double2) * 10 * (size_t)N;
-      e = cudaFuncSetAttribute(k_pd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) k_pd<<<(unsigned)P2, kRowThreads, smem, st>>>(B, av, h, A, Q, R);
-    }
+    const size_t smem = sizeof(double2) * 10 * (size_t)N;
+    e = cudaFuncSetAttribute(k_pd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) k_pd<<<(unsigned)P2, kRowThreads, smem, st>>>(B, av, h, A, Q, R);
     note_launch(1);
   }
   mark(2);
-  // 2: diagonal x pair (closed: produced by k_shared_closed below)
-  if (dense_out && !closed && e == cudaSuccess) {
+  // 2: diagonal x pair
+  if (dense_out && e == cudaSuccess) {
     k_dp<<<(unsigned)((N - 1) * chunks), 256, 0, st>>>(B, av, h, A, Q, R);
     note_launch(1);
   }
   mark(3);
-  // closed: stream-ordered scratch for the D x D tables (same edge), the vertex sums of K's
-  // diagonal rows and the diagonal x diagonal tables
-  double* scratch = nullptr;
-  const size_t dd_at = 3 * (size_t)N * N + N;
-  if (closed && e == cudaSuccess && (dense_out || K)) {
-    // from the retained pool: after a synchronization the default one would go to the driver again (0.15 ms)
-    cudaMemPool_t pool = nullptr;
-    if ((e = scratch_pool(&pool)) == cudaSuccess)
-      e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch),
-                                  sizeof(double) * (dd_at + DDTables::doubles(N)), pool, st);
-  }
-  // 3: diagonal x diagonal (closed: cells of constant coefficient from row,
-  //    column and corner sums)
-  if (dense_out && e == cudaSuccess && N >= 2) {
-    if (closed) {
-      const DDTables T = DDTables::carve(scratch + dd_at, N);
-      const int cols = 2 * N + 2 * (N + 1);
-      const int64_t ents = (int64_t)(N - 1) * (N - 1);
-      k_dd_rows<<<(unsigned)N, 128, 0, st>>>(B, av, T);
-      k_dd_cols<<<(unsigned)((cols + 127) / 128), 128, 0, st>>>(B, T);
-      k_dd_cells<<<(unsigned)((ents + 255) / 256), 256, 0, st>>>(B, T, A, Q, R);
-      note_launch(3);
-    } else {
-      const int64_t dd_warps = (int64_t)(N - 1) * (N - 1);
-      k_dd<<<(unsigned)((dd_warps * 32 + 255) / 256), 256, 0, st>>>(B, av, A, Q, R);
-      note_launch(1);
-    }
+  // 3: diagonal x diagonal
+  if (dense_out && e == cudaSuccess) {
+    const int64_t dd_warps = (int64_t)(N - 1) * (N - 1);
+    k_dd<<<(unsigned)((dd_warps * 32 + 255) / 256), 256, 0, st>>>(B, av, A, Q, R);
+    note_launch(1);
   }
   mark(4);
-  // 4: pair x pair on edges sharing one vertex (join: adds to R / A);
-  //    closed: one block per vertex pair writes these entries whole (the
-  //    D-section and Q parts too) and the diagonal x pair entries
-  if (dense_out && closed && e == cudaSuccess) {
-    const size_t smem = sizeof(double) * 32 * (size_t)(N + 1);
-    e = cudaFuncSetAttribute(k_shared_closed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_shared_closed<<<(unsigned)B.P, 256, smem, st>>>(B, av, h, A, Q, R);
-    note_launch(1);
-  } else if ((A || R) && N >= 3 && e == cudaSuccess) {
+  // 4: pair x pair on edges sharing one vertex (adds to R / A)
+  if ((A || R) && N >= 3 && e == cudaSuccess) {
     const size_t smem = sizeof(double2) * 6 * (size_t)N;
     e = cudaFuncSetAttribute(k_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) k_shared<<<(unsigned)(N * (N - 1)), 256, smem, st>>>(B, av, A, R);
     note_launch(1);
   }
   mark(5);
-  // 5: pair x pair on the same edge (closed: written whole, Q included; join:
-  //    adds to R / A); its D-section sums come from H = D X D^T of the D x D
-  //    block of a (stream-ordered scratch)
-  if ((closed ? dense_out : (A || R)) && e == cudaSuccess) {
-    if (closed) {
-      double* CXr = scratch;                     // N x N
-      double* SXi = scratch + (size_t)N * N;     // (N + 1) x N
-      if (N >= 2) {
-        k_dtab<<<(unsigned)(N - 1), 128, 0, st>>>(B, av, CXr, SXi);
-        note_launch(1);
-      }
-      k_same_closed<<<(unsigned)B.P, kSameThreads, 0, st>>>(B, av, h, CXr, SXi, A, Q, R);
-      note_launch(1);
-    } else {
-      k_same<<<(unsigned)B.P, kSameThreads, sizeof(double) * 2 * N, st>>>(B, av, A, R);
-      note_launch(1);
-    }
+  // 5: pair x pair on the same edge (adds to R / A)
+  if ((A || R) && e == cudaSuccess) {
+    k_same<<<(unsigned)B.P, kSameThreads, sizeof(double) * 2 * N, st>>>(B, av, A, R);
+    note_launch(1);
   }
   mark(6);
-  // 6: K (closed: the diagonal rows from the vertex sums G in the scratch)
+  // 6: K
   if (K && e == cudaSuccess) {
-    if (closed) {
-      // the pair rows of K come from k_pd_closed when it runs
-      const int64_t warps = 2 * B.P;
-      if (warps > 0 && !dense_out) {
-        k_kvec<true><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(B, av, K);
-        note_launch(1);
-      }
-      double* G = scratch + 3 * (size_t)N * N;
-      k_kvec_diag_g<<<(unsigned)N, 128, 0, st>>>(B, av, G);
-      k_kvec_diag<<<1, 256, 0, st>>>(B, G, K);
-      note_launch(2);
-    } else {
-      const int64_t warps = B.M;
-      k_kvec<false><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(B, av, K);
-      note_launch(1);
-    }
+    k_kvec<false><<<(unsigned)((B.M * 32 + 255) / 256), 256, 0, st>>>(B, av, K);
+    note_launch(1);
   }
   mark(7);
-  if (scratch) {
-    const cudaError_t ef = cudaFreeAsync(scratch, st);
-    if (e == cudaSuccess) e = ef;
-  }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -2668,9 +2740,10 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
 const char* assemble_kernel_name(int i) {
   static const char* names[kAssembleKernels] = {
       "k_entries (pair x pair; closed: disjoint edges by vertex quadruple)", "k_pd (pair x diagonal)",
-      "k_dp (diagonal x pair)", "k_dd (diagonal x diagonal)",
+      "k_dp (diagonal x pair)", "k_dd (diagonal x diagonal; closed: the tables)",
       "k_shared (edges sharing a vertex; closed: whole entries, + diagonal x pair)",
-      "k_same (same edge; closed: whole entries)", "k_kvec (K)"};
+      "k_same (same edge; closed: whole entries, + diagonal x diagonal, + K's diagonal rows)",
+      "k_kvec (K; closed: when only K is asked for)"};
   return (i >= 0 && i < kAssembleKernels) ? names[i] : nullptr;
 }
 

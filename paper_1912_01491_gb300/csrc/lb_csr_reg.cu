@@ -39,9 +39,6 @@ using lbi::CsrRegView;
 
 constexpr int kSkip = 255;  // length of a row that belongs to no group
 
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // A group's record: base (two words: the place of its values in the CSR arrays,
 // explicit: of its slots), L entries, kind (0 regular, 1 explicit).
 constexpr int kRec = 4;
@@ -271,10 +268,10 @@ __global__ void __launch_bounds__(stage_threads(PREC, TD), stage_blocks(PREC, TD
   const int lane = threadIdx.x & 31;
   const V* x = static_cast<const V*>(xv);
   V* xn = static_cast<V*>(xnv);
-  grid_release();
+  lb::grid_release();
   if (w < A.nlong) {
     const int64_t s = __ldg(A.longrow + w);
-    grid_wait();
+    lb::grid_wait();
     double y = as_double(long_row<V>(A, s, lane, x));
     if constexpr (TD) y = fma(eps, long_row<V>(Q1, s, lane, x), y);
     if (lane == 0) stage_row<STAGE>(s, y, Keff[s], v[s], STAGE > 1 ? acc[s] : 0.0, h, xn, acc, v);
@@ -287,7 +284,7 @@ __global__ void __launch_bounds__(stage_threads(PREC, TD), stage_blocks(PREC, TD
     int len = valid ? (int)__ldg(A.len8 + s) : 0;
     const bool mine = valid && len != kSkip;
     if (!mine) len = 0;
-    grid_wait();
+    lb::grid_wait();
     double kf = 0.0, vs = 0.0, ac = 0.0;
     if (mine) {
       kf = __ldcs(Keff + s);
@@ -303,7 +300,7 @@ __global__ void __launch_bounds__(stage_threads(PREC, TD), stage_blocks(PREC, TD
   if (s - lane >= M) return;  // whole warps leave together
   Group<V, 8> G;
   G.load(A, s >> 5, lane);
-  grid_wait();
+  lb::grid_wait();
   double kf = 0.0, vs = 0.0, ac = 0.0;
   if (s < M) {  // asked for before the group's kind is known; a regular group's rows all exist
     kf = __ldcs(Keff + s);

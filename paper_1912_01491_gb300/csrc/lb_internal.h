@@ -10,6 +10,16 @@
 #include "lindblad.h"
 #include "su_n.cuh"
 
+#if defined(__CUDACC__)
+namespace lb {
+// Kernels launched with programmatic stream serialization: the next grid may
+// start once every block has released it; wait until the grids before this one
+// are complete and their stores visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+}  // namespace lb
+#endif
+
 // Device-resident basis: the lexicographic pair table and the per-level
 // constants (layout of d_tab: c[N], lc[N], c2[N], inv[N+1]).
 struct lb_basis {
@@ -53,8 +63,8 @@ constexpr int kAssembleKernels = 7;
 // triangle crosses the link (one 2D copy per row block), the strict lower
 // triangle is then written on the device as a_kj = conj(a_jk).
 cudaError_t upload_hermitian(const double2* host, double2* dev, int64_t M, cudaStream_t st);
-// ev (kAssembleKernels + 1 events, optional): the kernels run in sequence
-// on st with an event between them.
+// ev (kAssembleKernels + 1 events, optional): the kernels run one after the
+// other on st with an event between them, else they overlap.
 cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double2* a,
                            double* A, double* Q, double* R, double* K, int algorithm, cudaStream_t st,
                            cudaEvent_t* ev = nullptr);
