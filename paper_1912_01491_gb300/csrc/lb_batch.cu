@@ -262,8 +262,7 @@ __global__ void __launch_bounds__(512, 2) k_rk4_batch(const BItem* __restrict__ 
         // FP64 defect c = (A64 - A32) v on own rows, with the full current v in x64
         for (int i = warp; i < nrow; i += nw) {
           const int64_t s = r0 + i;
-          double c = 0.0;
-          for (int n = lane; n < M; n += 32) c = fma(it.A64[s * M + n] - lb::widen(it.A32[s * M + n]), x64[n], c);
+          double c = lb::defect_dot<false>(it.A64 + s * M, it.A32 + s * M, 1.f, x64, M, lane);
           for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
           if (lane == 0) keff[i] = it.K[s] + c;
         }

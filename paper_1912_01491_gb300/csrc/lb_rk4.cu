@@ -191,24 +191,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   const int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= M) return;
-  const double* __restrict__ r64 = A64 + s * M;
-  double t = 0.0;
-  if (PREC == LB_FP32) {
-    const float* __restrict__ r = static_cast<const float*>(Ap) + s * M;
-    for (int64_t n = lane; n < M; n += 32) t = fma(__ldcs(r64 + n) - lb::widen(__ldcs(r + n)), v[n], t);
-  } else {
-    // sum_n A64_sn v_n - r_s sum_n q_sn v_n: two FP64 dot products (the
-    // difference is formed once per row, not per entry)
-    const uint16_t* __restrict__ r = static_cast<const uint16_t*>(Ap) + s * M;
-    double tq = 0.0;
-    for (int64_t n = lane; n < M; n += 32) {
-      const double vn = v[n];
-      t = fma(__ldcs(r64 + n), vn, t);
-      tq = fma(lb::widen(bf16_bits_to_float(__ldcs(reinterpret_cast<const unsigned short*>(r + n)))), vn, tq);
-    }
-    for (int o = 16; o > 0; o >>= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
-    if (lane == 0) t = fma(-(double)scale[s], tq, t);  // once, before the lane sum below
-  }
+  using E = typename std::conditional<PREC == LB_FP32, float, uint16_t>::type;
+  double t = lb::defect_dot<true>(A64 + s * M, static_cast<const E*>(Ap) + s * M, PREC == LB_BF16 ? scale[s] : 1.f, v,
+                            (int)M, lane);
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) Keff[s] = K[s] + t;
 }

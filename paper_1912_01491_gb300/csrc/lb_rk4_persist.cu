@@ -371,23 +371,10 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
 #pragma unroll 1
     for (int r = 0; r < R && i0 + r < nr; ++r) {
       const int sr = r0 + i0 + r;
-      const double* r64 = A.A64 + (int64_t)sr * M;
-      const E* rl = grows[0] + (size_t)r * M;
       double t = 0.0;
-      if constexpr (PREC == LB_FP32) {
-#pragma unroll 4
-        for (int n = lane; n < M; n += 32) t = fma(__ldcs(r64 + n) - lb::widen(rl[n]), x64[n], t);
-      } else if constexpr (PREC == LB_BF16) {
-        double tq = 0.0;
-#pragma unroll 4
-        for (int n = lane; n < M; n += 32) {
-          const double vn = x64[n];
-          t = fma(__ldcs(r64 + n), vn, t);
-          tq = fma(lb::widen(bf16_float(rl[n])), vn, tq);
-        }
-        for (int o = 16; o > 0; o >>= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
-        if (lane == 0) t = fma(-(double)A.scale[sr], tq, t);
-      }
+      if constexpr (!F64)
+        t = lb::defect_dot<false>(A.A64 + (int64_t)sr * M, grows[0] + (size_t)r * M, PREC == LB_BF16 ? A.scale[sr] : 1.f, x64,
+                           M, lane);
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       if (lane == r) kf = k0 + t;
     }
