@@ -50,6 +50,20 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t u) {
   return __uint_as_float(((uint32_t)u) << 16);
 }
 
+// FP32 stages: vectors of a row requested ahead, and the most warps an SM holds
+// (two blocks; 72 registers).
+constexpr int kAhead = 8, kStageWarps = 28;
+
+// An element of the matrix: read once, so it takes no place in L1, which the
+// four shifted copies of x need.
+__device__ __forceinline__ float4 load_once(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+
 template <int PREC>
 __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __restrict__ Ap,
                                           const float* __restrict__ scale,
@@ -78,33 +92,28 @@ __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __re
     const int64_t h4 = (int64_t)(((16 - ((uintptr_t)row & 15)) & 15) >> 2);
     const int head = (int)(h4 < M ? h4 : M);
     const int o = head & 3;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    if (lane < head) a0 = fmaf(__ldcs(row + lane), __ldg(x32 + lane), a0);
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+    if (lane < head) a[0] = fmaf(__ldcs(row + lane), __ldg(x32 + lane), a[0]);
     const float4* __restrict__ rv = reinterpret_cast<const float4*>(row + head);
     const float4* __restrict__ xv = reinterpret_cast<const float4*>(x32 + o * xstride + head - o);
-    const int64_t nv = (M - head) >> 2;
-    int64_t k = lane;
-    for (; k + 32 < nv; k += 64) {
-      const float4 u = __ldcs(rv + k), w = __ldcs(rv + k + 32);
-      const float4 xu = __ldg(xv + k), xw = __ldg(xv + k + 32);
-      a0 = fmaf(u.x, xu.x, a0);
-      a1 = fmaf(u.y, xu.y, a1);
-      a2 = fmaf(u.z, xu.z, a2);
-      a3 = fmaf(u.w, xu.w, a3);
-      a0 = fmaf(w.x, xw.x, a0);
-      a1 = fmaf(w.y, xw.y, a1);
-      a2 = fmaf(w.z, xw.z, a2);
-      a3 = fmaf(w.w, xw.w, a3);
+    const int nv = (int)((M - head) >> 2);
+    for (int k = lane; k < nv; k += 32 * kAhead) {
+      float4 u[kAhead];
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i)
+        if (k + 32 * i < nv) u[i] = load_once(rv + k + 32 * i);
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        if (k + 32 * i < nv) {
+          const float4 xu = __ldg(xv + k + 32 * i);
+          a[0] = fmaf(u[i].x, xu.x, a[0]);
+          a[1] = fmaf(u[i].y, xu.y, a[1]);
+          a[2] = fmaf(u[i].z, xu.z, a[2]);
+          a[3] = fmaf(u[i].w, xu.w, a[3]);
+        }
+      }
     }
-    for (; k < nv; k += 32) {
-      const float4 u = __ldcs(rv + k), xu = __ldg(xv + k);
-      a0 = fmaf(u.x, xu.x, a0);
-      a1 = fmaf(u.y, xu.y, a1);
-      a2 = fmaf(u.z, xu.z, a2);
-      a3 = fmaf(u.w, xu.w, a3);
-    }
-    for (int64_t n = head + 4 * nv + lane; n < M; n += 32) a0 = fmaf(__ldcs(row + n), __ldg(x32 + n), a0);
-    const float a[4] = {a0, a1, a2, a3};
+    for (int64_t n = head + 4 * (int64_t)nv + lane; n < M; n += 32) a[0] = fmaf(__ldcs(row + n), __ldg(x32 + n), a[0]);
     return lb::lane_sum(a);
   } else {
     // BF16: lane k reads four values (8 bytes) of A at element head + 4k
@@ -153,13 +162,17 @@ __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __re
   }
 }
 
+// FP32, us a stage with two vectors ahead, blocks of eight warps and plain
+// streaming loads, and now: M = 6399 37.1 / 29.6, 9999 79.2 / 63.4, 16899 185.6 /
+// 163.2, 22499 342.9 / 290.6, 39999 982.6 / 877.7 (7.29 TB/s).  BF16 gains
+// nothing from either: twice the bytes of x for those of A make it L1's.
 template <int PREC, int STAGE>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(PREC == LB_FP32 ? kStageWarps * 16 : kWarpsPerBlock * 32, PREC == LB_FP32 ? 2 : 0)
     k_stage(int64_t M, const void* __restrict__ Ap, const float* __restrict__ scale,
             const double* __restrict__ Keff, const double* __restrict__ x,
             const float* __restrict__ x32, double* __restrict__ xn, float* __restrict__ xn32,
             int64_t xstride, double* __restrict__ acc, double* __restrict__ v, double h) {
-  const int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+  const int64_t s = (int64_t)blockIdx.x * (PREC == LB_FP32 ? (int)(blockDim.x >> 5) : kWarpsPerBlock) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= M) return;
   const double y = row_dot<PREC>(M, s, Ap, scale, x, x32, xstride, lane);
@@ -745,12 +758,29 @@ Work carve(void* base, int64_t M) {
   return w;
 }
 
+// Warps of a stage kernel's block.  FP32: two blocks an SM.  A row is a warp's,
+// and the rows of an SM go in rounds of up to kStageWarps; a last round with few
+// rows takes as long as a full one at a fraction of the memory rate, so the
+// warps are as many as make the rounds equal.
+int stage_block_warps(int64_t M, int prec) {
+  if (prec != LB_FP32) return kWarpsPerBlock;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return kWarpsPerBlock;
+  const int64_t rows = (M + sms - 1) / sms, rounds = (rows + kStageWarps - 1) / kStageWarps;
+  const int64_t warps = (rows + rounds - 1) / rounds;
+  return (int)((warps + 1) / 2);
+}
+
 template <int PREC>
 cudaError_t run_steps(int64_t M, const void* Ap, const float* scale, const double* A64,
                       int correct_every, const double* K, double* v, double dt, int64_t nsteps,
                       double* snaps, int64_t snap_every, const Work& w, cudaStream_t st) {
   const unsigned grid = (unsigned)((M + kWarpsPerBlock - 1) / kWarpsPerBlock);
   const unsigned bs = kWarpsPerBlock * 32;
+  const int sw = stage_block_warps(M, PREC);
+  const unsigned sgrid = (unsigned)((M + sw - 1) / sw), sbs = 32u * (unsigned)sw;
   cudaError_t e;
   e = cudaMemcpyAsync(w.X, v, sizeof(double) * M, cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return e;
@@ -767,10 +797,10 @@ cudaError_t run_steps(int64_t M, const void* Ap, const float* scale, const doubl
       k_correction<PREC><<<grid, bs, 0, st>>>(M, A64, Ap, scale, v, K, w.Keff);
       lbi::note_launch(1);
     }
-    k_stage<PREC, 1><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, 0.5 * dt);
-    k_stage<PREC, 2><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, 0.5 * dt);
-    k_stage<PREC, 3><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
-    k_stage<PREC, 4><<<grid, bs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt / 6.0);
+    k_stage<PREC, 1><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, 0.5 * dt);
+    k_stage<PREC, 2><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, 0.5 * dt);
+    k_stage<PREC, 3><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
+    k_stage<PREC, 4><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt / 6.0);
     lbi::note_launch(4);
     if (snaps && snap_every > 0 && (t + 1) % snap_every == 0) {
       e = cudaMemcpyAsync(snaps + ((t + 1) / snap_every - 1) * M, v, sizeof(double) * M,

@@ -49,3 +49,27 @@ def test_sum_of_partial_sums(m, precision, gap):
         want, size = 6.0 * math.fsum(row), math.fsum(abs(x) for x in row)
         bound = 4 * eps * abs(want) + (6 * 8 * eps * size if gap > 29 else 0.0)
         assert abs(v[s].item() - want) <= bound, (s, v[s].item(), want)
+
+
+@pytest.mark.parametrize("M", [4257, 9001])
+def test_stage_rows_in_rounds(M):
+    """FP32 stages of more rows than an SM takes at once (one launch per stage,
+    M = 4257 rows: one full round; 9001: three): one step against FP64 with the
+    same FP32 matrix.  Each of the four stages adds at most (M + 4) 2^-24 of
+    w = |A| |x| + |K| to its slope, x = v + dt k with |dt k| <= 2 dt w; factor 2
+    to spare."""
+    import paper_1912_01491_gb300 as lb
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    A = (torch.randn((M, M), generator=gen, device="cuda") / M ** 0.5).contiguous()
+    K = torch.randn(M, generator=gen, device="cuda", dtype=torch.float64) / M
+    v0 = torch.randn(M, generator=gen, device="cuda", dtype=torch.float64)
+    dt, A64, v = 1e-3, A.double(), v0.clone()
+    lb.rk4_dense(A, K, v, dt, 1, precision="fp32", work=lb.rk4_workspace(M))
+    k1 = A64 @ v0 + K
+    k2 = A64 @ (v0 + 0.5 * dt * k1) + K
+    k3 = A64 @ (v0 + 0.5 * dt * k2) + K
+    k4 = A64 @ (v0 + dt * k3) + K
+    ref = v0 + dt / 6 * (k1 + 2 * k2 + 2 * k3 + k4)
+    w = A64.abs() @ v0.abs() + K.abs()
+    bound = 2 * dt * (M + 4) * 2.0 ** -24 * (w + 2 * dt * (A64.abs() @ w)) + 2.0 ** -51 * v0.abs()
+    assert bool(((v - ref).abs() <= bound).all())
