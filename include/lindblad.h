@@ -612,8 +612,9 @@ int lb_integrate(lb_system_t *sys, int precision, int correct_every, const doubl
                  int64_t snap_every, double *v_out);
 
 /* Return the spare device memory of the library pool of the current device
- * (after the library stream has finished).  The next host-buffer call
- * reserves again what it needs. */
+ * (after the library stream has finished), and that of the pool the
+ * assemblies take their scratch and sparse systems their arrays from (up to
+ * 2 GiB kept between calls).  The next call reserves again what it needs. */
 int lb_host_release(void);
 
 /* Checkpoint and resume.  There is no counterpart in the paper; it serves
