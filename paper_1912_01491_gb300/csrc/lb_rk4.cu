@@ -50,6 +50,7 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t u) {
   return __uint_as_float(((uint32_t)u) << 16);
 }
 
+constexpr int kFewWarps = 20;  // BF16: blocks of 20 warps, two an SM, in place of six of eight
 // FP32 stages: vectors of a row requested ahead, and the most warps an SM holds
 // (two blocks; 72 registers).
 constexpr int kAhead = 8, kStageWarps = 28;
@@ -166,13 +167,13 @@ __device__ __forceinline__ double row_dot(int64_t M, int64_t s, const void* __re
 // streaming loads, and now: M = 6399 37.1 / 29.6, 9999 79.2 / 63.4, 16899 185.6 /
 // 163.2, 22499 342.9 / 290.6, 39999 982.6 / 877.7 (7.29 TB/s).  BF16 gains
 // nothing from either: twice the bytes of x for those of A make it L1's.
-template <int PREC, int STAGE>
-__global__ void __launch_bounds__(PREC == LB_FP32 ? kStageWarps * 16 : kWarpsPerBlock * 32, PREC == LB_FP32 ? 2 : 0)
+template <int PREC, int STAGE, bool FEW = false>
+__global__ void __launch_bounds__(PREC == LB_FP32 ? kStageWarps * 16 : FEW ? 32 * kFewWarps : kWarpsPerBlock * 32, PREC == LB_FP32 || FEW ? 2 : 0)
     k_stage(int64_t M, const void* __restrict__ Ap, const float* __restrict__ scale,
             const double* __restrict__ Keff, const double* __restrict__ x,
             const float* __restrict__ x32, double* __restrict__ xn, float* __restrict__ xn32,
             int64_t xstride, double* __restrict__ acc, double* __restrict__ v, double h) {
-  const int64_t s = (int64_t)blockIdx.x * (PREC == LB_FP32 ? (int)(blockDim.x >> 5) : kWarpsPerBlock) + (threadIdx.x >> 5);
+  const int64_t s = (int64_t)blockIdx.x * (PREC == LB_FP32 ? (int)(blockDim.x >> 5) : FEW ? kFewWarps : kWarpsPerBlock) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= M) return;
   const double y = row_dot<PREC>(M, s, Ap, scale, x, x32, xstride, lane);
@@ -762,12 +763,19 @@ Work carve(void* base, int64_t M) {
 // and the rows of an SM go in rounds of up to kStageWarps; a last round with few
 // rows takes as long as a full one at a fraction of the memory rate, so the
 // warps are as many as make the rounds equal.
+// BF16, bound by L1 more than by loads under way: 48 warps an SM, or 40 where
+// their rounds come out a tenth fuller (us a stage, 48 / 40: M = 9999 45.1 / 44.4,
+// 16899 102.0 / 101.0, 22499 188 / 183).
 int stage_block_warps(int64_t M, int prec) {
-  if (prec != LB_FP32) return kWarpsPerBlock;
+  if (prec == LB_FP64) return kWarpsPerBlock;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return kWarpsPerBlock;
+  if (prec == LB_BF16) {
+    const double r48 = (double)M / (48 * sms), r40 = (double)M / (40 * sms);  // rounds
+    return r48 > 1.25 && r40 / std::ceil(r40) > 1.1 * r48 / std::ceil(r48) ? kFewWarps : kWarpsPerBlock;
+  }
   const int64_t rows = (M + sms - 1) / sms, rounds = (rows + kStageWarps - 1) / kStageWarps;
   const int64_t warps = (rows + rounds - 1) / rounds;
   return (int)((warps + 1) / 2);
@@ -792,15 +800,25 @@ cudaError_t run_steps(int64_t M, const void* Ap, const float* scale, const doubl
   }
   const bool correct = PREC != LB_FP64 && correct_every > 0 && A64 != nullptr;
   const int64_t xs = w.xstride;
+  auto stage = [&](auto n, auto... args) {
+    constexpr int S = decltype(n)::value;
+    if constexpr (PREC == LB_BF16) {
+      if (sw == kFewWarps) {
+        k_stage<PREC, S, true><<<sgrid, sbs, 0, st>>>(args...);
+        return;
+      }
+    }
+    k_stage<PREC, S><<<sgrid, sbs, 0, st>>>(args...);
+  };
   for (int64_t t = 0; t < nsteps; ++t) {
     if (correct && t % correct_every == 0) {
       k_correction<PREC><<<grid, bs, 0, st>>>(M, A64, Ap, scale, v, K, w.Keff);
       lbi::note_launch(1);
     }
-    k_stage<PREC, 1><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, 0.5 * dt);
-    k_stage<PREC, 2><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, 0.5 * dt);
-    k_stage<PREC, 3><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
-    k_stage<PREC, 4><<<sgrid, sbs, 0, st>>>(M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt / 6.0);
+    stage(std::integral_constant<int, 1>{}, M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, 0.5 * dt);
+    stage(std::integral_constant<int, 2>{}, M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, 0.5 * dt);
+    stage(std::integral_constant<int, 3>{}, M, Ap, scale, w.Keff, w.X, w.X32, w.Y, w.Y32, xs, w.acc, v, dt);
+    stage(std::integral_constant<int, 4>{}, M, Ap, scale, w.Keff, w.Y, w.Y32, w.X, w.X32, xs, w.acc, v, dt / 6.0);
     lbi::note_launch(4);
     if (snaps && snap_every > 0 && (t + 1) % snap_every == 0) {
       e = cudaMemcpyAsync(snaps + ((t + 1) / snap_every - 1) * M, v, sizeof(double) * M,
