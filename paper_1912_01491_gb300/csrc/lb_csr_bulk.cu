@@ -414,7 +414,9 @@ __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk 
   // candidate counts of at most 4 x 4 take 16 lanes a pair
   if ((*b.maxdeg <= 4) != (GW == 16)) return;
   const unsigned long long lim = mag_bits(1e-12 * *b.smax);
-  const bool cplx = *b.cplx != 0;
+  // no bound: every row goes the general way, those whose entries all cancel too (under a negative bound the join
+  // keeps even zeros)
+  const bool bounded = lim < 0x7ff0000000000000ull, cplx = *b.cplx != 0;
   unsigned long long nterm = 0;
   for (int64_t w0 = (blockIdx.x * (int64_t)256 + (threadIdx.x & ~31)) / GW; w0 < B.P;
        w0 += gridDim.x * (int64_t)256 / GW) {
@@ -427,8 +429,8 @@ __global__ void __launch_bounds__(256) k_bulk_rows(BasisView B, int nP, CsrBulk 
     d = e.b;
   }
   const int dc = b.deg[c], dd = b.deg[d];
-  bool bulk = in && (FILL ? !b.slow[pr] : !b.near[(int64_t)c * N + d] && !b.near[(int64_t)d * N + c] && dc > 0 &&
-                                              dd > 0 && dc * dd <= GW);
+  bool bulk = in && (FILL ? !b.slow[pr] : bounded && !b.near[(int64_t)c * N + d] && !b.near[(int64_t)d * N + c] &&
+                                              dc > 0 && dd > 0 && dc * dd <= GW);
   double re = 0.0, im = 0.0;
   bool kre = false, kim = false, unsure = false, flip = false;
   int32_t pi = 0x7fffffff;
