@@ -234,7 +234,13 @@ size_t lb_rk4_workspace_bytes(int64_t M);
  * v (M doubles) is the initial state on entry and the final state on exit.
  * snaps (may be NULL): after every snap_every steps a copy of v is stored in
  * row t/snap_every - 1 of snaps ((nsteps/snap_every) x M).
- * work: lb_rk4_workspace_bytes(M) bytes of device memory. */
+ * work: lb_rk4_workspace_bytes(M) bytes of device memory.
+ * M <= 3600 (LB_FP32: 3400), not under stream capture: all steps are one
+ * cooperative launch whose blocks exchange the stage vector and wait for one
+ * another, each wait for some two seconds of clock at most.  The call is
+ * asynchronous, so it returns before a wait can run out; the rows that depend
+ * on it are then NaN in v and in the snapshots, all others are right.
+ * (lb_integrate, which is synchronous, returns LB_ETIMEOUT.) */
 int lb_rk4_dense(int64_t M, int precision, const void *Ap, const float *row_scale,
                  const double *A64, int correct_every, const double *K, double *v,
                  double dt, int64_t nsteps, double *snaps, int64_t snap_every,
@@ -607,7 +613,8 @@ int lb_system_get_csr(const lb_system_t *sys, int64_t *rowptr, int32_t *col, dou
  * for lb_rk4_dense; the low-precision copy is made (and cached in the
  * system) on first use.  CSR systems: LB_FP64 or LB_FP32 as for lb_rk4_csr;
  * with LB_FP32 and correct_every > 0, snap_every must be a multiple of
- * correct_every (the correction restarts at every snapshot).  Synchronous. */
+ * correct_every (the correction restarts at every snapshot).  Synchronous.
+ * LB_ETIMEOUT, v_out untouched, if a bounded wait of the kernels ran out. */
 int lb_integrate(lb_system_t *sys, int precision, int correct_every, const double *v0, double t, double dt,
                  int64_t snap_every, double *v_out);
 

@@ -1240,9 +1240,17 @@ static int integrate_steps(lb_system_t* s, int precision, int correct_every, con
                     "snapshot");
     }
   } else {
+    const int* waits = nullptr;
     LB_TRY_CUDA(lbi::rk4_dense(M, precision, Ap, s->scale, s->A, correct_every, s->K, dv.as<double>(), dt, n,
-                               nsnap > 0 ? dsn.as<double>() : nullptr, nsnap > 0 ? snap_every : 0, work.p, c.st),
+                               nsnap > 0 ? dsn.as<double>() : nullptr, nsnap > 0 ? snap_every : 0, work.p, c.st, true,
+                               &waits),
                 "RK4");
+    if (waits) {  // before v_out is written
+      int flag = 0;
+      LB_TRY_CUDA(cudaMemcpyAsync(&flag, waits, sizeof(int), cudaMemcpyDeviceToHost, c.st), "RK4: waits");
+      LB_TRY_CUDA(cudaStreamSynchronize(c.st), "lb_integrate");
+      if (flag) return lbi::cuda_fail(cudaErrorLaunchTimeout, "lb_integrate: a wait between the blocks of a step ran out");
+    }
   }
   if (nsnap > 0)
     LB_TRY_CUDA(cudaMemcpyAsync(v_out, dsn.p, 8 * (size_t)M * nsnap, cudaMemcpyDeviceToHost, c.st), "copy snapshots");

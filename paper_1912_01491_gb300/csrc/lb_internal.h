@@ -174,10 +174,12 @@ cudaError_t rk4_csr_td(int64_t M, const int64_t* rowptr, const int32_t* col, con
 cudaError_t pack_fp32(int64_t M, const double* A, float* A32, cudaStream_t st);
 cudaError_t pack_bf16(int64_t M, const double* A, uint16_t* Ab, float* scale, cudaStream_t st);
 size_t rk4_workspace_bytes(int64_t M);
+// waits (optional): null, or when the steps have bounded waits (one launch) the
+// device flag that is nonzero after the steps if one ran out.
 cudaError_t rk4_dense(int64_t M, int precision, const void* Ap, const float* scale,
                       const double* A64, int correct_every, const double* K, double* v,
                       double dt, int64_t nsteps, double* snaps, int64_t snap_every,
-                      void* work, cudaStream_t st, bool one_launch = true);
+                      void* work, cudaStream_t st, bool one_launch = true, const int** waits = nullptr);
 // All steps in one cooperative launch (lb_rk4_persist.cu), bit-identical to
 // the stage launches: whether the size is in its range, and the launch
 // (*done = false: not taken, nothing enqueued).  ll: 32 M bytes, keff: M

@@ -1097,8 +1097,9 @@ size_t rk4_workspace_bytes(int64_t M) {
 cudaError_t rk4_dense(int64_t M, int precision, const void* Ap, const float* scale,
                       const double* A64, int correct_every, const double* K, double* v, double dt,
                       int64_t nsteps, double* snaps, int64_t snap_every, void* work,
-                      cudaStream_t st, bool one_launch) {
+                      cudaStream_t st, bool one_launch, const int** waits) {
   Work w = carve(work, M);
+  if (waits) *waits = nullptr;
   if (one_launch && nsteps > 0 && rk4_persist_applies(M, precision)) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cap);
@@ -1106,6 +1107,7 @@ cudaError_t rk4_dense(int64_t M, int precision, const void* Ap, const float* sca
     if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone)
       e = rk4_persist(M, precision, Ap, scale, A64, correct_every, K, v, dt, nsteps, snaps, snap_every, w.Keff, w.X32,
                       w.err, st, &done);
+    if (done && waits) *waits = w.err;
     if (e != cudaSuccess || done) return e;
   }
   switch (precision) {

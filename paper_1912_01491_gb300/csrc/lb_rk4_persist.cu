@@ -17,8 +17,10 @@
 // it has polled every element of stage g + 1, and a block sends those only
 // after it has read all of stage g: no reader can lag behind.  The launch is
 // cooperative (all blocks are resident) and every poll is bounded (about two
-// seconds of clock): a block whose poll runs out goes on without waiting and
-// writes NaN to its rows of v, so the failure shows.
+// seconds of clock).  A block whose poll runs out sets *err, waits no more and
+// takes NaN for every element that has not come: each row reads all of x, so all
+// of its rows are NaN from the next stage on, and so are those of a block that
+// still takes its words.  An element of v or of a snapshot is either right or NaN.
 //
 // Arithmetic: the row sums are those of k_stage (FP64: the same lane order and
 // shuffle tree; FP32 and BF16: the same 128 partial sums, summed by
@@ -36,6 +38,8 @@ namespace {
 
 constexpr long long kPollCycles = 4000000000LL;
 constexpr int kMaxWarps = 16;
+
+thread_local long long t_poll_cycles = kPollCycles;
 
 struct PersistArgs {
   int M, nr, rem;  // rows per block: nr, the first rem blocks one more
@@ -55,6 +59,7 @@ struct PersistArgs {
   unsigned long long* ll;  // two buffers of bufw words
   size_t bufw;
   int* err;
+  long long poll_cycles;
 };
 
 __device__ __forceinline__ void ll_store(unsigned long long* p, uint32_t data, uint32_t flag) {
@@ -332,13 +337,14 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
       };
       auto wait = [&](int q) {
         while (!ready(q) && !bad()) {
-          if (clock64() - c0 > kPollCycles) {
+          if (clock64() - c0 > A.poll_cycles) {
             dead = 1;
             atomicExch(A.err, 1);
             break;
           }
           ll_load2(buf + 2 * (p0 + q * nthr), w[q][0], w[q][1]);
         }
+        if (!ready(q)) w[q][0] = w[q][1] = 0x7ff80000u;  // NaN: FP32, and the high word of FP64
       };
       ll_load2(buf + 2 * p0, w[0][0], w[0][1]);
       wait(0);
@@ -446,7 +452,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
   }
   __syncthreads();
   if (holds) {
-    A.v[s] = bad() ? __longlong_as_double(0x7ff8000000000000LL) : vs;
+    A.v[s] = vs;
     A.keff_out[s] = kf;
   }
 }
@@ -513,6 +519,7 @@ cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* s
   a.ll = static_cast<unsigned long long*>(ll);
   a.bufw = 2 * (size_t)M;
   a.err = err;
+  a.poll_cycles = t_poll_cycles;
   const void* f = f64 ? pick<LB_FP64>(R) : precision == LB_FP32 ? pick<LB_FP32>(R) : pick<LB_BF16>(R);
   // warps without rows still poll
   const int threads = M <= 300 ? 256 : 32 * kMaxWarps;
@@ -527,7 +534,7 @@ cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* s
     a.nsteps = std::min(chunk, nsteps - t);
     a.keff0 = t ? keff : nullptr;
     e = cudaMemsetAsync(ll, 0, 16 * a.bufw, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
+    if (e == cudaSuccess && t == 0) e = cudaMemsetAsync(err, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     void* params[] = {&a};
     e = cudaLaunchCooperativeKernel(f, dim3((unsigned)G), dim3((unsigned)threads), params, smem, st);
@@ -543,3 +550,11 @@ cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* s
 }
 
 }  // namespace lbi
+
+// For tests, not part of the ABI: the limit in clock cycles of one poll in this
+// thread's later calls (negative: give up where a word has not come yet); returns the previous one.
+extern "C" long long lbi_poll_cycles(long long cycles) {
+  const long long before = t_poll_cycles;
+  t_poll_cycles = cycles;
+  return before;
+}
