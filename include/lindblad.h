@@ -240,7 +240,11 @@ size_t lb_rk4_workspace_bytes(int64_t M);
  * another, each wait for some two seconds of clock at most.  The call is
  * asynchronous, so it returns before a wait can run out; the rows that depend
  * on it are then NaN in v and in the snapshots, all others are right.
- * (lb_integrate, which is synchronous, returns LB_ETIMEOUT.) */
+ * (lb_integrate, which is synchronous, returns LB_ETIMEOUT.)  Such a launch
+ * holds its SMs until its last step, and starts when all of them have room:
+ * up to N of about 36 (LB_FP64) or 48 launches of several streams share the
+ * chip, larger ones run one after the other, and other work on those SMs with
+ * much shared memory or many registers waits for them. */
 int lb_rk4_dense(int64_t M, int precision, const void *Ap, const float *row_scale,
                  const double *A64, int correct_every, const double *K, double *v,
                  double dt, int64_t nsteps, double *snaps, int64_t snap_every,

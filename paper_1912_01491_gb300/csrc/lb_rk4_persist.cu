@@ -457,6 +457,24 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
   }
 }
 
+// Warps of a block; those without rows still poll.  No more than the rows need:
+// a block of 16 takes all registers of an SM, and then the launches of several
+// streams run one after the other.  us a step of all, 16 warps / now / with a
+// launch per stage, 8 streams: FP32 N = 20 89 / 26 / 42, N = 30 101 / 25 / 48,
+// N = 36 96 / 47 / 55, N = 44 109 / 62 / 92, FP64 N = 20 81 / 39 / 43, N = 30 137 / 92 /
+// 69; one stream: FP32 N = 20 11.4 / 7.9, N = 30 13.8 / 8.8, N = 33 8.4 / 9.8, N = 44
+// 13.9 / 11.4, FP64 N = 30 18.5 / 14.4 (fewer pollers leave L2 to the stores).
+// FP64 rows are a warp's time each: two a warp cost more than they free (N = 40,
+// one stream: 28 / 42).  Where a launch needs the shared memory of all SMs (FP64
+// N >= 38, FP32 N >= 49) the streams still run one after the other: 8 streams of
+// FP32 N = 50 128 against 119 with a launch per stage, FP64 532 against 389.
+int block_warps(int64_t M, int nrows, bool f64) {
+  if (M <= 200) return 8;
+  if (nrows <= 4) return 4;
+  if (f64) return nrows <= 8 ? 8 : kMaxWarps;
+  return nrows <= 8 ? 4 : nrows <= 16 ? 8 : kMaxWarps;
+}
+
 template <int PREC>
 const void* pick(int R) {
   return R == 1 ? (const void*)k_rk4_persist<PREC, 1> : (const void*)k_rk4_persist<PREC, 2>;
@@ -496,8 +514,9 @@ cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* s
   a.nr = (int)(M / G);
   a.rem = (int)(M % G);
   const int nrows = a.nr + (a.rem ? 1 : 0);
-  const int R = nrows > kMaxWarps ? 2 : 1;  // one round of rows: their state stays in registers
-  if (nrows > R * kMaxWarps) return cudaSuccess;
+  const int warps = block_warps(M, nrows, f64);
+  const int R = nrows > warps ? 2 : 1;  // one round of rows: their state stays in registers
+  if (nrows > R * warps) return cudaSuccess;
   a.xpad = (int)((M + 127) & ~int64_t(127)) + 32;  // the first lanes read up to 32 past the end
   a.pitch = f64 ? (int)((M + 31) & ~int64_t(31)) : (int)((M + 127) & ~int64_t(127));
   const bool correct = !f64 && correct_every > 0 && A64 != nullptr;
@@ -521,8 +540,7 @@ cudaError_t rk4_persist(int64_t M, int precision, const void* Ap, const float* s
   a.err = err;
   a.poll_cycles = t_poll_cycles;
   const void* f = f64 ? pick<LB_FP64>(R) : precision == LB_FP32 ? pick<LB_FP32>(R) : pick<LB_BF16>(R);
-  // warps without rows still poll
-  const int threads = M <= 300 ? 256 : 32 * kMaxWarps;
+  const int threads = 32 * warps;
   e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
   int per = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, threads, smem);
