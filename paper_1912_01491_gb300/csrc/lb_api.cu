@@ -109,6 +109,7 @@ struct lb_system {
   uint16_t* Abf = nullptr;
   float* scale = nullptr;
   lbi::CsrOut csr;               // LB_CSR: rowptr, col, val, K (K aliases csr.K)
+  std::mutex mu;                 // held while an integration makes what the system keeps of a CSR matrix
   float* csr32 = nullptr;        // FP32 copy of csr.val, made on first use
   lbi::CsrPlan plan;             // layout of a CSR system, made on first use
   double ms[LB_PHASES] = {};     // phase times of the call that built it
@@ -1190,18 +1191,18 @@ static int integrate_steps(lb_system_t* s, int precision, int correct_every, con
   const void* Ap = s->format == LB_CSR ? (const void*)s->csr.val : (const void*)s->A;
   lbi::CsrRegView view;
   bool reg = false;
-  if (s->format == LB_CSR)
+  if (s->format == LB_CSR) {
+    std::lock_guard<std::mutex> lock(s->mu);
     LB_TRY_CUDA(csr_view(s->csr, &s->plan, precision, c.st, &view, &reg), "lb_integrate: layout");
-  if (reg) {
-    // the layout holds the values
-  } else if (precision == LB_FP32 && s->format == LB_CSR) {
-    if (!s->csr32) {
-      DevBuf b32;
-      if ((rc = alloc_or_enomem(b32, sizeof(float) * (size_t)(s->csr.nnz + 1), "FP32 values")) != LB_OK) return rc;
-      LB_TRY_CUDA(lbi::to_f32(s->csr.nnz, s->csr.val, b32.as<float>(), c.st), "pack FP32 values");
-      s->csr32 = static_cast<float*>(b32.release());
+    if (!reg && precision == LB_FP32) {  // else the layout holds the values
+      if (!s->csr32) {
+        DevBuf b32;
+        if ((rc = alloc_or_enomem(b32, sizeof(float) * (size_t)(s->csr.nnz + 1), "FP32 values")) != LB_OK) return rc;
+        LB_TRY_CUDA(lbi::to_f32(s->csr.nnz, s->csr.val, b32.as<float>(), c.st), "pack FP32 values");
+        s->csr32 = static_cast<float*>(b32.release());
+      }
+      Ap = s->csr32;
     }
-    Ap = s->csr32;
   } else if (precision == LB_FP32) {
     if (!s->A32) {
       PoolBuf b32;
