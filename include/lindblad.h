@@ -624,8 +624,8 @@ int lb_integrate(lb_system_t *sys, int precision, int correct_every, const doubl
 
 /* Return the spare device memory of the library pool of the current device
  * (after the library stream has finished), and that of the pool the
- * assemblies take their scratch and sparse systems their arrays from (up to
- * 2 GiB kept between calls).  The next call reserves again what it needs. */
+ * assemblies take their scratch from (up to 2 GiB kept between calls).  The
+ * next call reserves again what it needs. */
 int lb_host_release(void);
 
 /* Checkpoint and resume.  There is no counterpart in the paper; it serves

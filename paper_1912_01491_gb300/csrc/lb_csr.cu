@@ -926,11 +926,13 @@ inline unsigned nb(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 namespace lbi {
 
-// The scratch pool of a device: temporaries of the assemblies, and the arrays
-// of sparse systems.  It keeps up to kScratchKeep between calls (a cudaMalloc or
-// cudaFree of the sizes here takes 0.1 to several ms and synchronizes the
-// device; the ladder at N = 2000 spent 10 of its 41 ms in them), the rest goes
-// back at the next synchronization, all of it with lb_host_release.
+// The scratch pool of a device: temporaries of the assemblies.  It keeps up to
+// kScratchKeep between calls (a cudaMalloc or cudaFree of the sizes here takes
+// 0.1 to several ms and synchronizes the device; the ladder at N = 2000 spent 10
+// of its 41 ms in them), the rest goes back at the next synchronization, all of
+// it with lb_host_release.  The arrays of a system do not come from it: pool
+// memory is not visible to other devices and cannot be exported, and it is freed
+// without waiting for the kernels that read it.
 constexpr uint64_t kScratchKeep = uint64_t(2) << 30, kLargeScratch = uint64_t(1) << 29;
 
 cudaError_t scratch_pool(cudaMemPool_t* out) {
@@ -962,8 +964,6 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
 }
 
 void csr_out_free(CsrOut* m) {
-  if (!m->rowptr) return;
-  cudaDeviceSynchronize();  // kernels of any stream may still read the arrays
   cudaFree(m->rowptr);
   cudaFree(m->col);
   cudaFree(m->val);
@@ -987,11 +987,12 @@ struct Buf {
     else if (p) cudaFreeAsync(p, st);
     p = nullptr;
   }
+  cudaError_t alloc_own(size_t n) {  // outlives the call
+    large = true;
+    return cudaMalloc(&p, n);
+  }
   cudaError_t alloc(size_t n) {
-    if (n > kLargeScratch) {
-      large = true;
-      return cudaMalloc(&p, n);
-    }
+    if (n > kLargeScratch) return alloc_own(n);
     cudaMemPool_t pool = nullptr;
     const cudaError_t e = scratch_pool(&pool);
     return e == cudaSuccess ? cudaMallocFromPoolAsync(&p, n ? n : 16, pool, st) : e;
@@ -1206,15 +1207,15 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   CK(rows_long(k_rows_long<kLongThreads>, kLongThreads, nlong, longlist.as<int64_t>() + (rows - nlong), kLongCap));
   CK(rows_long(k_rows_long<kMidThreads>, kMidThreads, nmid, longlist.as<int64_t>(), 2 * kMidBound));
   Buf rowptr(st);
-  CK(rowptr.alloc(sizeof(int64_t) * (size_t)(M + 1)));
+  CK(rowptr.alloc_own(sizeof(int64_t) * (size_t)(M + 1)));
   int64_t nnz = 0;
   CK(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
   CK(scan_counts(rowc.as<unsigned long long>(), rowptr.as<int64_t>(), M, &nnz, st));
   if (hc[2] != 0) return cudaErrorNotSupported;  // a row has more than kLongCap distinct columns
   Buf col(st), val(st), K(st);
-  CK(col.alloc(sizeof(int32_t) * (size_t)(nnz + 1)));
-  CK(val.alloc(sizeof(double) * (size_t)(nnz + 1)));
-  CK(K.alloc(sizeof(double) * (size_t)M));
+  CK(col.alloc_own(sizeof(int32_t) * (size_t)(nnz + 1)));
+  CK(val.alloc_own(sizeof(double) * (size_t)(nnz + 1)));
+  CK(K.alloc_own(sizeof(double) * (size_t)M));
   k_rows_copy<<<std::max(nb(rows, 8), 1u), 256, 0, st>>>(rows, I.list, tmpoff.as<int64_t>(), tcol.as<int32_t>(),
                                                          tval.as<double>(), rowptr.as<int64_t>(), col.as<int32_t>(), val.as<double>());
   note_launch(1);

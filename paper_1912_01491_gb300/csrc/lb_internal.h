@@ -115,9 +115,8 @@ cudaError_t csr_bulk_count(const lb::BasisView& B, const CsrBulk& b, int nP, con
                            unsigned long long* nlist, cudaStream_t st);
 cudaError_t csr_bulk_fill(const lb::BasisView& B, const CsrBulk& b, int nP, const int64_t* rowptr, int32_t* col,
                           double* val, cudaStream_t st);
-// The device's scratch pool (stream-ordered temporaries and the CsrOut arrays).
+// The device's scratch pool (stream-ordered temporaries).
 cudaError_t scratch_pool(cudaMemPool_t* out);
-// Frees the arrays; waits for the device first.
 void csr_out_free(CsrOut* m);
 cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP, const double* gamma_host,
                                  const int64_t* lp_ptr_host, const int64_t* lp_idx, const double2* lp_val,
