@@ -350,16 +350,8 @@ cudaError_t launch(int stage, const cudaLaunchConfig_t& cfg, int64_t M, const Cs
 namespace lbi {
 
 void csr_plan_free(CsrPlan* p) {
-  cudaFree(p->rec);
-  cudaFree(p->delta);
-  cudaFree(p->len8);
-  cudaFree(p->ecol);
-  cudaFree(p->longrow);
-  cudaFree(p->egroup);
-  for (int q = 0; q < 2; ++q) {
-    cudaFree(p->val[q]);
-    cudaFree(p->eval[q]);
-  }
+  cudaFree(p->rec);  // with the arrays behind it
+  for (int q = 0; q < 2; ++q) cudaFree(p->val[q]);
   *p = CsrPlan{};
 }
 
@@ -370,10 +362,8 @@ cudaError_t csr_plan(CsrPlan* p, int64_t M, int64_t nnz, const int64_t* rowptr, 
   cudaError_t e = cudaSuccess;
   const int64_t groups = (M + 31) / 32;
   const unsigned grid = nblk(groups * 32);
+  auto pad = [](size_t n) { return (n + 255) & ~size_t(255); };
   // without memory for it the caller takes the kernels that need no layout
-  auto alloc = [&](auto** q, size_t n) {
-    if (e == cudaSuccess) e = cudaMalloc((void**)q, n);
-  };
   auto refused = [&]() {
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
@@ -382,25 +372,35 @@ cudaError_t csr_plan(CsrPlan* p, int64_t M, int64_t nnz, const int64_t* rowptr, 
   if (p->state == 0) {
     unsigned long long *cnt = nullptr, hc[3] = {0, 0, 0};
     const int longer = (int)std::min<int64_t>(200, 8 + 5 * nnz / (4 * M));
-    alloc(&cnt, sizeof(hc));
-    if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(hc), st);
+    cudaMemPool_t pool = nullptr;
+    if ((e = scratch_pool(&pool)) != cudaSuccess) return e;
+    if ((e = cudaMallocFromPoolAsync((void**)&cnt, sizeof(hc), pool, st)) != cudaSuccess) return refused();
+    e = cudaMemsetAsync(cnt, 0, sizeof(hc), st);
     if (e == cudaSuccess) {
       k_reg_desc<false><<<grid, 256, 0, st>>>(M, longer, rowptr, col, cnt, nullptr, nullptr, nullptr, nullptr, nullptr,
                                               nullptr);
-          note_launch(1);
+      note_launch(1);
       e = cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     // padding or long rows without end: the CSR kernels
     const bool fits = 2 * hc[0] <= 3ull * (unsigned long long)nnz + 4096 && 8 * (int64_t)hc[1] <= M;
     if (e == cudaSuccess && fits) {
-      alloc(&p->rec, sizeof(int32_t) * kRec * (size_t)groups);
-      alloc(&p->delta, sizeof(int32_t) * (size_t)(nnz / 32 + 1));
-      alloc(&p->len8, (size_t)M);
-      alloc(&p->ecol, sizeof(int32_t) * (size_t)(hc[0] + 1));
-      alloc(&p->longrow, sizeof(int32_t) * (size_t)(hc[1] + 1));
-      alloc(&p->egroup, sizeof(int32_t) * (size_t)(hc[2] + 1));
-      if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(hc), st);
+      // one allocation: each takes some ten microseconds whatever its size
+      const size_t rec = pad(sizeof(int32_t) * kRec * (size_t)groups), delta = pad(sizeof(int32_t) * (size_t)(nnz / 32 + 1)),
+                   len8 = pad((size_t)M), ecol = pad(sizeof(int32_t) * (size_t)(hc[0] + 1)),
+                   longrow = pad(sizeof(int32_t) * (size_t)(hc[1] + 1)), egroup = sizeof(int32_t) * (size_t)(hc[2] + 1);
+      char* m = nullptr;
+      e = cudaMalloc((void**)&m, rec + delta + len8 + ecol + longrow + egroup);
+      if (e == cudaSuccess) {
+        p->rec = reinterpret_cast<int32_t*>(m);
+        p->delta = reinterpret_cast<int32_t*>(m += rec);
+        p->len8 = reinterpret_cast<uint8_t*>(m += delta);
+        p->ecol = reinterpret_cast<int32_t*>(m += len8);
+        p->longrow = reinterpret_cast<int32_t*>(m += ecol);
+        p->egroup = reinterpret_cast<int32_t*>(m += longrow);
+        e = cudaMemsetAsync(cnt, 0, sizeof(hc), st);
+      }
       if (e == cudaSuccess) {
         k_reg_desc<true><<<grid, 256, 0, st>>>(M, longer, rowptr, col, cnt, p->rec, p->delta, p->len8, p->ecol,
                                                p->longrow, p->egroup);
@@ -408,7 +408,7 @@ cudaError_t csr_plan(CsrPlan* p, int64_t M, int64_t nnz, const int64_t* rowptr, 
         e = cudaStreamSynchronize(st);
       }
     }
-    cudaFree(cnt);
+    cudaFreeAsync(cnt, st);
     if (e != cudaSuccess || !fits) {
       csr_plan_free(p);
       if (e == cudaSuccess) p->state = -1;
@@ -421,25 +421,23 @@ cudaError_t csr_plan(CsrPlan* p, int64_t M, int64_t nnz, const int64_t* rowptr, 
   }
   const int q = precision == LB_FP64 ? 0 : 1;
   if (!p->val[q]) {
-    void *a = nullptr, *b = nullptr;
-    const size_t esz = q == 0 ? 8 : 4;
-    alloc(&a, esz * (size_t)(nnz + 8));
-    alloc(&b, esz * (size_t)(p->slots + 1));
+    const size_t esz = q == 0 ? 8 : 4, first = pad(esz * (size_t)(nnz + 8));
+    char* a = nullptr;
+    e = cudaMalloc((void**)&a, first + esz * (size_t)(p->slots + 1));
     if (e == cudaSuccess) {
       if (q == 0)
-        k_reg_values<double><<<grid, 256, 0, st>>>(M, p->rec, p->len8, rowptr, val, (double*)a, (double*)b);
+        k_reg_values<double><<<grid, 256, 0, st>>>(M, p->rec, p->len8, rowptr, val, (double*)a, (double*)(a + first));
       else
-        k_reg_values<float><<<grid, 256, 0, st>>>(M, p->rec, p->len8, rowptr, val, (float*)a, (float*)b);
+        k_reg_values<float><<<grid, 256, 0, st>>>(M, p->rec, p->len8, rowptr, val, (float*)a, (float*)(a + first));
       note_launch(1);
       e = cudaStreamSynchronize(st);  // other streams use it from here on
     }
     if (e != cudaSuccess) {
       cudaFree(a);
-      cudaFree(b);
       return refused();
     }
     p->val[q] = a;
-    p->eval[q] = b;
+    p->eval[q] = a + first;
   }
   *view = CsrRegView{p->rec, p->delta, p->len8, p->ecol, p->longrow, p->egroup, p->nlong, p->nexp,
                      p->val[q], p->eval[q], nnz,

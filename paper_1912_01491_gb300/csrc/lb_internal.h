@@ -128,9 +128,9 @@ cudaError_t to_f32(int64_t n, const double* x, float* y, cudaStream_t st);
 struct CsrPlan {
   int state = 0;  // 0: not looked at, 1: made, -1: the pattern does not suit it
   int64_t slots = 0, nlong = 0, nexp = 0;
-  int32_t *rec = nullptr, *delta = nullptr, *ecol = nullptr, *longrow = nullptr, *egroup = nullptr;
-  uint8_t* len8 = nullptr;
-  void *val[2] = {nullptr, nullptr}, *eval[2] = {nullptr, nullptr};  // FP64, FP32
+  int32_t *rec = nullptr, *delta = nullptr, *ecol = nullptr, *longrow = nullptr, *egroup = nullptr;  // one allocation
+  uint8_t* len8 = nullptr;                                                                           // (rec)
+  void *val[2] = {nullptr, nullptr}, *eval[2] = {nullptr, nullptr};  // FP64, FP32: val and eval one allocation
 };
 struct CsrRegView {
   const int32_t *rec, *delta;
