@@ -2542,13 +2542,18 @@ cudaError_t upload_hermitian(const double2* host, double2* dev, int64_t M, cudaS
   return cudaGetLastError();
 }
 
+// The dynamic shared memory that the dense kernels may ask for: what the largest
+// N needs, the same from every thread.  A limit of the call's own size could be
+// lowered by a call with a smaller N on another thread before the launch.
+constexpr int kMostShared = (int)sizeof(double) * 32 * (kMaxDenseN + 1);
+
 // Launch behind what is queued on st; overlap: the grids before it may still
 // run (they have all released it, and it waits where it reads what they write).
 template <class... P, class... X>
 static cudaError_t launch_on(bool overlap, void (*kernel)(P...), int64_t grid, int threads, size_t smem,
                              cudaStream_t st, X... x) {
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostShared);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg{};
@@ -2695,7 +2700,7 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
   // 1: pair x diagonal
   if (dense_out && e == cudaSuccess) {
     const size_t smem = sizeof(double2) * 10 * (size_t)N;
-    e = cudaFuncSetAttribute(k_pd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_pd, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostShared);
     if (e == cudaSuccess) k_pd<<<(unsigned)P2, kRowThreads, smem, st>>>(B, av, h, A, Q, R);
     note_launch(1);
   }
@@ -2716,7 +2721,7 @@ cudaError_t assemble_dense(const lb::BasisView& B, const double* h, const double
   // 4: pair x pair on edges sharing one vertex (adds to R / A)
   if ((A || R) && N >= 3 && e == cudaSuccess) {
     const size_t smem = sizeof(double2) * 6 * (size_t)N;
-    e = cudaFuncSetAttribute(k_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_shared, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostShared);
     if (e == cudaSuccess) k_shared<<<(unsigned)(N * (N - 1)), 256, smem, st>>>(B, av, A, R);
     note_launch(1);
   }
@@ -2758,3 +2763,15 @@ cudaError_t join_terms(const lb::BasisView& B, unsigned long long* d_count, cuda
 }
 
 }  // namespace lbi
+
+// For tests, not part of the ABI: the least of the limits of the kernels above
+// whose need grows past the default with N (bytes of dynamic shared memory; < 0: a CUDA error).
+extern "C" int lbi_dense_shared_limit(int join) {
+  cudaFuncAttributes a{}, b{};
+  if (join) {
+    if (cudaFuncGetAttributes(&a, k_pd) != cudaSuccess || cudaFuncGetAttributes(&b, k_shared) != cudaSuccess) return -1;
+    return a.maxDynamicSharedSizeBytes < b.maxDynamicSharedSizeBytes ? a.maxDynamicSharedSizeBytes
+                                                                     : b.maxDynamicSharedSizeBytes;
+  }
+  return cudaFuncGetAttributes(&a, k_shared_closed) == cudaSuccess ? a.maxDynamicSharedSizeBytes : -1;
+}

@@ -872,6 +872,7 @@ cudaError_t run_steps_csr(int64_t M, const int64_t* rowptr, const int32_t* col, 
   // buffers of it stay within 112 KB (chunks above the capacity are summed
   // from global memory)
   int pcap = 0;
+  const int lim = (int)((56 * 1024 - kPipeRowBytes) / (sizeof(V) + sizeof(int32_t))) - 16;
   if (pipe) {
     e = cudaMemsetAsync(w.err, 0, sizeof(int), st);
     if (e == cudaSuccess) {
@@ -880,7 +881,6 @@ cudaError_t run_steps_csr(int64_t M, const int64_t* rowptr, const int32_t* col, 
       int mx = 0;
       e = cudaMemcpyAsync(&mx, w.err, sizeof(int), cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      const int lim = (int)((56 * 1024 - kPipeRowBytes) / (sizeof(V) + sizeof(int32_t))) - 16;
       pcap = ((mx < lim ? mx : lim) + 7) & ~7;
     }
     if (e != cudaSuccess) return e;
@@ -892,10 +892,12 @@ cudaError_t run_steps_csr(int64_t M, const int64_t* rowptr, const int32_t* col, 
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     if (pipe) {
-      attr((const void*)k_stage_csr_pipe<PREC, 1>, psmem);
-      attr((const void*)k_stage_csr_pipe<PREC, 2>, psmem);
-      attr((const void*)k_stage_csr_pipe<PREC, 3>, psmem);
-      attr((const void*)k_stage_csr_pipe<PREC, 4>, psmem);
+      // the largest of any system: another thread's call sets the same
+      const size_t most = 2 * csr_pipe_buf_bytes<V>((lim + 7) & ~7);
+      attr((const void*)k_stage_csr_pipe<PREC, 1>, most);
+      attr((const void*)k_stage_csr_pipe<PREC, 2>, most);
+      attr((const void*)k_stage_csr_pipe<PREC, 3>, most);
+      attr((const void*)k_stage_csr_pipe<PREC, 4>, most);
       int dev = 0, sms = 0, per = 0;
       if (e == cudaSuccess) e = cudaGetDevice(&dev);
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -904,10 +906,10 @@ cudaError_t run_steps_csr(int64_t M, const int64_t* rowptr, const int32_t* col, 
       const int64_t nch = (M + 255) / 256, resident = (int64_t)sms * (per > 0 ? per : 1);
       pgrid = (unsigned)(nch < resident ? nch : resident);
     } else {
-      attr((const void*)k_stage_csr_blk<PREC, 1>, smem);
-      attr((const void*)k_stage_csr_blk<PREC, 2>, smem);
-      attr((const void*)k_stage_csr_blk<PREC, 3>, smem);
-      attr((const void*)k_stage_csr_blk<PREC, 4>, smem);
+      attr((const void*)k_stage_csr_blk<PREC, 1>, 48 * 1024);  // csr_stage_cap's bound
+      attr((const void*)k_stage_csr_blk<PREC, 2>, 48 * 1024);
+      attr((const void*)k_stage_csr_blk<PREC, 3>, 48 * 1024);
+      attr((const void*)k_stage_csr_blk<PREC, 4>, 48 * 1024);
     }
     if (e != cudaSuccess) return e;
   }
