@@ -484,6 +484,9 @@ int lb_csr_copy(const lb_csr_t* c, int64_t* rowptr, int32_t* col, double* val, d
   return LB_OK;
 }
 
+// For tests, not part of the ABI: rows that the assembly summed by the join.
+long long lbi_csr_joined(const lb_csr_t* c) { return c->m.joined; }
+
 int lb_csr_destroy(lb_csr_t* c) {
   if (!c) return LB_OK;
   lbi::csr_out_free(&c->m);

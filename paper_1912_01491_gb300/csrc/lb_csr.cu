@@ -1242,6 +1242,7 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   out->K = K.as<double>();
   K.p = nullptr;
   out->terms = nterms + (int64_t)hb[0];
+  out->joined = rows;
   return cudaSuccess;
 }
 

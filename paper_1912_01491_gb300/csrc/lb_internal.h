@@ -74,6 +74,7 @@ cudaError_t join_terms(const lb::BasisView& B, unsigned long long* d_count, cuda
 // sparse assembly (lb_csr.cu)
 struct CsrOut {
   int64_t M = 0, nnz = 0, terms = 0;
+  int64_t joined = 0;         // rows summed by the join, the others in closed form
   int64_t* rowptr = nullptr;  // M + 1
   int32_t* col = nullptr;     // nnz, sorted within rows
   double* val = nullptr;      // nnz
