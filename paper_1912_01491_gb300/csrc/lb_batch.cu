@@ -721,9 +721,15 @@ int smem_optin() {
 }
 
 // Shared-memory layout for (mmax, C): as many rows as fit; total 0 if not even
-// the vectors do.
+// the vectors do.  FP64 slices that do not fit whole leave room for a second
+// block on the SM (an SM then takes two realizations, and one's FP64 sums run
+// beside the other's loads and barriers): 30 steps, one block / two, the best
+// cluster size, 32 of N = 33, 35 14.5 / 12.3 ms, 48 of N = 36 26.4 / 20.8, 48 of
+// N = 40 43.0 / 31.3, 16 of N = 64 equal.  In FP32 the rows held are worth more
+// (48 of N = 40 8.6 / 13.3).
 SmemLayout pick_layout(int64_t mmax, int C, size_t es) {
-  const size_t cap = (size_t)smem_optin();
+  constexpr size_t kReserved = 1024;  // of an SM's shared memory, a block
+  size_t cap = (size_t)smem_optin();
   SmemLayout L = layout(mmax, C, true, es);
   if (L.total <= cap) return L;
   L = layout(mmax, C, false, es);
@@ -731,6 +737,8 @@ SmemLayout pick_layout(int64_t mmax, int C, size_t es) {
     L.total = 0;
     return L;
   }
+  const size_t half = (cap + kReserved) / 2 - kReserved;
+  if (es == sizeof(double) && L.total <= half) cap = half;
   L.room = (int64_t)((cap - L.total) / es);
   L.total = cap;
   return L;
@@ -745,8 +753,10 @@ SmemLayoutP pick_layoutP(int64_t mmax, int C, bool f64) {
 }
 
 // Threads of a block of k_rk4_batch: where the shared memory leaves room for
-// one block an SM, 16 warps keep enough loads under way.
-int rk4_threads(size_t smem) { return 2 * smem > (size_t)smem_optin() ? 512 : 256; }
+// one block an SM, or rows are streamed, 16 warps keep enough loads under way.
+int rk4_threads(const SmemLayout& L) {
+  return 2 * L.total > (size_t)smem_optin() || L.room < L.slice * L.mmax ? 512 : 256;
+}
 
 // Launch configuration of a batched kernel (func) for n items at cluster size
 // C with smem bytes of dynamic shared memory; the number of clusters is what
@@ -859,7 +869,7 @@ cudaError_t batch_launch_group(lb_batch* b, const std::vector<int>& ids, int C, 
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   auto kernel = f64 ? k_rk4_batch<double> : k_rk4_batch<float>;
-  cudaError_t e = configure((const void*)kernel, C, L.total, (int)ids.size(), rk4_threads(L.total), st, &cfg, attr);
+  cudaError_t e = configure((const void*)kernel, C, L.total, (int)ids.size(), rk4_threads(L), st, &cfg, attr);
   if (e != cudaSuccess) return e;
   // items in decreasing order of work (largest first)
   std::vector<int> ord(ids.begin(), ids.end());
@@ -981,7 +991,7 @@ cudaError_t batch_launch_async(const BatchItem* items, int n, int C, int64_t nst
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   cudaError_t e =
-      configure((const void*)k_rk4_batch<float>, C, L.total, n, rk4_threads(L.total), st, &cfg, attr);
+      configure((const void*)k_rk4_batch<float>, C, L.total, n, rk4_threads(L), st, &cfg, attr);
   if (e != cudaSuccess) return e;
   std::vector<int> ord(n);
   for (int i = 0; i < n; ++i) ord[i] = i;
