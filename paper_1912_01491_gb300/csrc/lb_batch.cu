@@ -120,6 +120,35 @@ __device__ __forceinline__ void rows_dot(const T* const (&row)[R], const T* __re
   }
 }
 
+// The same for long rows that are streamed: eight elements of every row are asked
+// for before the first is used.
+template <class T, int W, int R>
+__device__ __forceinline__ void rows_dot_ahead(const T* const (&row)[R], const T* __restrict__ x, int M, int sub,
+                                               T (&a)[R]) {
+  constexpr int U = 8;
+#pragma unroll
+  for (int r = 0; r < R; ++r) a[r] = T(0);
+  int n = sub;
+  for (; n + (U - 1) * W < M; n += U * W) {
+    T e[R][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int r = 0; r < R; ++r) e[r][u] = __ldg(row[r] + n + u * W);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const T xn = x[n + u * W];
+#pragma unroll
+      for (int r = 0; r < R; ++r) a[r] = mad(e[r][u], xn, a[r]);
+    }
+  }
+  for (; n < M; n += W) {
+    const T xn = x[n];
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[r] = mad(row[r][n], xn, a[r]);
+  }
+}
+
 // Sums of R rows over the W lanes of each group.  The additions of a row are
 // those of the xor tree from W / 2 down; halves of the group take different
 // rows, so four rows cost 6 shuffles in place of 20.  Row r is then with the
@@ -159,7 +188,7 @@ __device__ __forceinline__ T rows_sum(const T (&a)[3], int sub) {
 }
 
 // Sums A x of the rows u G + g, u = u0, u0 + step, .. (R of them) of n, into sums.
-template <class T, int W, int R>
+template <class T, int W, int R, bool AHEAD = false>
 __device__ __forceinline__ void rows_batch(const T* __restrict__ mat, int n, int u0, int step,
                                            const T* __restrict__ x, int M, int lane, T* __restrict__ sums) {
   constexpr int G = 32 / W, parts = R == 1 ? 1 : R == 2 ? 2 : 4;
@@ -168,7 +197,8 @@ __device__ __forceinline__ void rows_batch(const T* __restrict__ mat, int n, int
 #pragma unroll
   for (int r = 0; r < R; ++r) row[r] = mat + (int64_t)min((u0 + r * step) * G + g, n - 1) * M;
   T a[R];
-  rows_dot<T, W, R>(row, x, M, sub, a);
+  if constexpr (AHEAD) rows_dot_ahead<T, W, R>(row, x, M, sub, a);
+  else rows_dot<T, W, R>(row, x, M, sub, a);
   const T t = rows_sum<T, W>(a, sub);
   const int r = sub / (W / parts), i = (u0 + r * step) * G + g;
   if (sub % (W / parts) == 0 && r < R && i < n) sums[i] = t;
@@ -190,6 +220,25 @@ __device__ __forceinline__ void rows_stage(const T* __restrict__ mat, int n, con
     else rows_batch<T, W, 1>(mat, n, u, nw, x, M, lane, sums);
     u += r * nw;
     left -= r;
+  }
+}
+
+// The same for streamed rows of systems from M = kLongRow on: at most two rows a
+// warp, eight elements of each ahead.  From N = 48 on the matrices of the clusters
+// under way exceed L2, and four rows a warp with what the compiler asks for ahead
+// left too few loads under way (30 steps, four rows / now: 16 of N = 64 69.7 /
+// 42.1 ms, 24 of N = 48, 50 22.8 / 18.6; FP64, 16 of N = 64 126 / 100); below N = 44
+// they are in L2, where four rows are quicker (48 of N = 40 8.6 / 9.4).
+constexpr int kLongRow = 1900;
+
+template <class T, int W>
+__device__ __forceinline__ void rows_far(const T* __restrict__ mat, int n, const T* __restrict__ x, int M, int w, int nw,
+                                         int lane, T* __restrict__ sums) {
+  constexpr int G = 32 / W;
+  int left = ((n + G - 1) / G - w + nw - 1) / nw;
+  for (int u = w; left > 0; u += 2 * nw, left -= 2) {
+    if (left >= 2) rows_batch<T, W, 2, true>(mat, n, u, nw, x, M, lane, sums);
+    else rows_batch<T, W, 1, true>(mat, n, u, nw, x, M, lane, sums);
   }
 }
 
@@ -218,7 +267,9 @@ __device__ __forceinline__ const double* matrix_of(const BItem& it, double) { re
 // N = 26 .. 28 29.5 -> 13.2 ms, 256 of N = 10 .. 12 3.2 -> 1.0 ms; FP64, 64 of
 // N = 33 .. 35 91 -> 85 ms, 256 of N = 18 .. 20 50 -> 35 ms (with one row a warp,
 // its epilogue on every lane, and a slice held whole or not at all).
-template <class T>
+// LONG: for groups with a system of M >= kLongRow (a kernel of its own: with both
+// forms in one, the others lost 4-7%).
+template <class T, bool LONG>
 __global__ void __launch_bounds__(512, 2) k_rk4_batch(const BItem* __restrict__ items, const int* __restrict__ order,
                                                       int nitems, int* __restrict__ counter, int64_t nsteps, double dt,
                                                       int correct_every, SmemLayout L) {
@@ -275,7 +326,9 @@ __global__ void __launch_bounds__(512, 2) k_rk4_batch(const BItem* __restrict__ 
         auto products = [&](auto width) {
           constexpr int W = decltype(width)::value;
           auto streamed = [&] {
-            rows_stage<T, W>(mat + (int64_t)held * M, nrow - held, xc, M, warp, nw, lane, sums + held);
+            const T* far = mat + (int64_t)held * M;
+            if constexpr (LONG) rows_far<T, W>(far, nrow - held, xc, M, warp, nw, lane, sums + held);
+            else rows_stage<T, W>(far, nrow - held, xc, M, warp, nw, lane, sums + held);
           };
           // every second warp begins with the streamed rows, so that shared memory and L2 are both busy
           if (warp & 1) streamed();
@@ -752,6 +805,11 @@ SmemLayoutP pick_layoutP(int64_t mmax, int C, bool f64) {
   return L;
 }
 
+template <class T>
+auto rk4_kernel(int64_t mmax) {
+  return mmax >= kLongRow ? k_rk4_batch<T, true> : k_rk4_batch<T, false>;
+}
+
 // Threads of a block of k_rk4_batch: where the shared memory leaves room for
 // one block an SM, or rows are streamed, 16 warps keep enough loads under way.
 int rk4_threads(const SmemLayout& L) {
@@ -868,7 +926,7 @@ cudaError_t batch_launch_group(lb_batch* b, const std::vector<int>& ids, int C, 
   if (L.total == 0) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  auto kernel = f64 ? k_rk4_batch<double> : k_rk4_batch<float>;
+  auto kernel = f64 ? rk4_kernel<double>(mmax) : rk4_kernel<float>(mmax);
   cudaError_t e = configure((const void*)kernel, C, L.total, (int)ids.size(), rk4_threads(L), st, &cfg, attr);
   if (e != cudaSuccess) return e;
   // items in decreasing order of work (largest first)
@@ -990,8 +1048,8 @@ cudaError_t batch_launch_async(const BatchItem* items, int n, int C, int64_t nst
   if (L.total == 0) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  cudaError_t e =
-      configure((const void*)k_rk4_batch<float>, C, L.total, n, rk4_threads(L), st, &cfg, attr);
+  auto kernel = rk4_kernel<float>(mmax);
+  cudaError_t e = configure((const void*)kernel, C, L.total, n, rk4_threads(L), st, &cfg, attr);
   if (e != cudaSuccess) return e;
   std::vector<int> ord(n);
   for (int i = 0; i < n; ++i) ord[i] = i;
@@ -1007,7 +1065,7 @@ cudaError_t batch_launch_async(const BatchItem* items, int n, int C, int64_t nst
   unsigned char* db = static_cast<unsigned char*>(d);
   e = cudaMemcpyAsync(d, host.data(), host.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
-    e = cudaLaunchKernelEx(&cfg, k_rk4_batch<float>, reinterpret_cast<const BItem*>(db),
+    e = cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const BItem*>(db),
                            reinterpret_cast<const int*>(db + off_o), n, reinterpret_cast<int*>(db + off_c), nsteps,
                            dt, correct_every, L);
   note_launch(1);
