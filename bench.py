@@ -736,6 +736,39 @@ def csr_step_bytes(precision, nnz, M):
     return 4.0 * per_stage + 8.0 * M + 48.0 * M
 
 
+def csr_layout_step_bytes(precision, rowptr, col):
+    """Algorithmic bytes of one RK4 step (4 stages) on the layout by groups of
+    32 rows (numpy CSR arrays).  Regular group (rows of equal length, entry j
+    of every row at the row plus one offset): its values, one set of offsets
+    and a record of 16 bytes.  Explicit group: values, columns, the rows'
+    lengths, its number, and its record twice (by its own warp and by the one
+    that finds it is not regular).  Long rows (more than 8 + 5/4 of the mean,
+    at most 200): FP64 values, columns, two row pointers and their number.
+    Vectors as in csr_step_bytes."""
+    import numpy as np
+    M, nnz = len(rowptr) - 1, int(rowptr[-1])
+    val = x = 4.0 if precision == "fp32" else 8.0
+    lens = np.diff(rowptr)
+    is_long = lens > min(200, 8 + 5 * nnz // (4 * M))
+    whole = M // 32
+    reg = np.zeros((M + 31) // 32, bool)
+    L = lens[:32 * whole].reshape(whole, 32)
+    same = (L == L[:, :1]).all(1) & ~is_long[:32 * whole].reshape(whole, 32).any(1)
+    for n in np.unique(L[same, 0]):
+        g = np.flatnonzero(same & (L[:, 0] == n))
+        for part in np.array_split(g, max(1, len(g) * 32 * int(n) >> 24)):
+            at = rowptr[32 * part][:, None, None] + np.arange(32 * n).reshape(1, 32, n)
+            d = col[at].astype(np.int64) - (32 * part[:, None, None] + np.arange(32).reshape(1, 32, 1))
+            reg[part] = (d == d[:, :1]).all((1, 2))
+    row_reg = np.repeat(reg, 32)[:M]
+    e_reg, e_long = float(lens[row_reg].sum()), float(lens[is_long].sum())
+    e_exp = nnz - e_reg - e_long
+    n_exp, n_long = float((~reg).sum()), float(is_long.sum())
+    per_stage = (e_reg * (val + 4.0 / 32) + 16.0 * len(reg) + e_exp * (val + 4.0) + n_exp * (16.0 + 4.0 + 32.0) +
+                 e_long * 12.0 + n_long * 20.0 + M * (x + 8.0 + 8.0 + x))
+    return 4.0 * per_stage + 8.0 * M + 48.0 * M
+
+
 def form_sparse(args, dev):
     """Sparse ladder model: CSR assembly of Q + R and K, CSR RK4 (FP32 values
     with FP64 correction every 50 steps, and FP64)."""
@@ -773,7 +806,8 @@ def form_sparse(args, dev):
         torch.cuda.synchronize()
         res[prec] = ev[0].elapsed_time(ev[1])
     nnz = c.nnz
-    step_bytes = {p: csr_step_bytes(p, nnz, M) for p in ("fp32", "fp64")}
+    rowptr, col = c.to_host()[:2]
+    step_bytes = {p: csr_layout_step_bytes(p, rowptr, col) for p in ("fp32", "fp64")}
     peaks = measured_peaks()
     hbm = peaks.get("hbm_gbs")
     gbs = {p: step_bytes[p] * n / (res[p] * 1e-3) / 1e9 for p in res}
@@ -781,11 +815,13 @@ def form_sparse(args, dev):
     B.close()
     return {"N": N, "M": M, "nnz": nnz, "row_terms": c.terms, "assembly_s": t_asm,
             "rk4_fp32c_steps_per_s": n / (res["fp32"] * 1e-3), "rk4_fp64_steps_per_s": n / (res["fp64"] * 1e-3),
-            "rk4_roofline": {"kernel": "k_stage_reg (CSR SpMV + stage update by groups of 32 rows with one set of column offsets; the bytes are those of the CSR form, the columns and row pointers of which it does not read)", "bound": "hbm",
+            "rk4_roofline": {"kernel": "k_stage_reg (SpMV + stage update by groups of 32 rows with one set of column offsets)",
+                             "bound": "hbm",
                              "achieved": gbs["fp32"], "peak": hbm, "unit": "GB/s",
                              "frac": gbs["fp32"] / hbm if hbm else None,
                              "algorithmic_bytes_per_step": step_bytes["fp32"],
-                             "fp64_achieved_gbs": gbs["fp64"]},
+                             "fp64_achieved_gbs": gbs["fp64"],
+                             "csr_form_bytes_per_step": csr_step_bytes("fp32", nnz, M)},
             "note": "FP32 row includes one FP64 correction SpMV every 50 steps in its time"}
 
 
