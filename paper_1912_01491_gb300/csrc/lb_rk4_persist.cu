@@ -461,17 +461,17 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
 // a block of 16 takes all registers of an SM, and then the launches of several
 // streams run one after the other.  us a step of all, 16 warps / now / with a
 // launch per stage, 8 streams: FP32 N = 20 89 / 26 / 42, N = 30 101 / 25 / 48,
-// N = 36 96 / 47 / 55, N = 44 109 / 62 / 92, FP64 N = 20 81 / 39 / 43, N = 30 137 / 92 /
+// N = 36 96 / 47 / 55, N = 44 109 / 62 / 92, FP64 N = 20 81 / 45 / 43, N = 30 137 / 92 /
 // 69; one stream: FP32 N = 20 11.4 / 7.9, N = 30 13.8 / 8.8, N = 33 8.4 / 9.8, N = 44
 // 13.9 / 11.4, FP64 N = 30 18.5 / 14.4 (fewer pollers leave L2 to the stores).
 // FP64 rows are a warp's time each: two a warp cost more than they free (N = 40,
-// one stream: 28 / 42).  Where a launch needs the shared memory of all SMs (FP64
+// one stream: 28 / 42), and so do four warps (N = 23 10.5 / 11.9) or eight for eight
+// rows (N = 34 17.9 / 20.8).  Where a launch needs the shared memory of all SMs (FP64
 // N >= 38, FP32 N >= 49) the streams still run one after the other: 8 streams of
 // FP32 N = 50 128 against 119 with a launch per stage, FP64 532 against 389.
 int block_warps(int64_t M, int nrows, bool f64) {
   if (M <= 200) return 8;
-  if (nrows <= 4) return 4;
-  if (f64) return nrows <= 8 ? 8 : kMaxWarps;
+  if (f64) return nrows <= 7 ? 8 : kMaxWarps;
   return nrows <= 8 ? 4 : nrows <= 16 ? 8 : kMaxWarps;
 }
 
