@@ -242,7 +242,7 @@ size_t lb_rk4_workspace_bytes(int64_t M);
  * on it are then NaN in v and in the snapshots, all others are right.
  * (lb_integrate, which is synchronous, returns LB_ETIMEOUT.)  Such a launch
  * holds its SMs until its last step, and starts when all of them have room:
- * up to N of about 36 (LB_FP64) or 48 launches of several streams share the
+ * up to N of about 32 (LB_FP64) or 48 launches of several streams share the
  * chip, larger ones run one after the other, and other work on those SMs with
  * much shared memory or many registers waits for them. */
 int lb_rk4_dense(int64_t M, int precision, const void *Ap, const float *row_scale,
@@ -364,8 +364,11 @@ typedef struct lb_csr lb_csr_t;
  * Eq. (09) is evaluated per channel as r_sn = -1/2 gamma_p Re sum_l W_ls U_ln,
  * U_ln = sum_j l_j z_jln, W_ls = sum_k conj(l_k) f_kls (a sparse product:
  * the terms are placed in buckets by row / column with count, scan and fill
- * passes, and each row of A is summed in a hash table keyed by column; the
+ * passes, and a row of A is summed in a hash table keyed by column; the
  * diagonal components of l_p and of h enter through closed-form edge sums).
+ * From N = 128 on, with at most four channels of rates >= 0, rows far from the
+ * diagonal on the graphs of the l_p and of H are formed from the matrix units
+ * instead, without these sums; the pattern rule and the pattern are the same.
  * Pattern: an entry is stored iff |A_sn| exceeds 1e-12 times the sum of the
  * magnitudes of its terms (exact cancellations leave rounding residue only);
  * columns are sorted within rows.  Values are reproducible to rounding (the
@@ -490,10 +493,10 @@ int lb_batch_form_propagator(lb_batch_t *b, double dt, void *stream, float *ms);
 
 /* RK4 for every realization, nsteps steps of dt, FP32 matrix with FP32
  * products, FP64 state, FP64 defect correction every correct_every steps (0:
- * none).  One persistent cluster launch per cluster-size group: a cluster
- * takes realizations from a queue (largest first), keeps its row slices of
- * the matrix in shared memory when they fit, and exchanges the stage
- * vector through distributed shared memory.  ms (optional) receives the
+ * none).  One persistent cluster launch per cluster-size group, the groups on
+ * streams of the batch behind `stream`: a cluster takes realizations from a
+ * queue (largest first), keeps as many rows of the matrix in shared memory as
+ * fit, and exchanges the stage vector through distributed shared memory.  ms (optional) receives the
  * device time.  Synchronous. */
 int lb_batch_integrate(lb_batch_t *b, int correct_every, double dt, int64_t nsteps, void *stream, float *ms);
 

@@ -264,9 +264,9 @@ __device__ __forceinline__ const double* matrix_of(const BItem& it, double) { re
 // matrix element and a quarter of x); rows streamed, L2.  At 40 levels a third
 // of the matrix fits a cluster of 16.  FP32, 100 steps at the best cluster size:
 // 48 of N = 39, 40 47.8 -> 23.1 ms, 64 of N = 33 .. 35 34.1 -> 18.1 ms, 128 of
-// N = 26 .. 28 29.5 -> 13.2 ms, 256 of N = 10 .. 12 3.2 -> 1.0 ms; FP64, 64 of
-// N = 33 .. 35 91 -> 85 ms, 256 of N = 18 .. 20 50 -> 35 ms (with one row a warp,
-// its epilogue on every lane, and a slice held whole or not at all).
+// N = 26 .. 28 29.5 -> 13.2 ms, 256 of N = 10 .. 12 3.2 -> 1.0 ms; FP64, 30 steps,
+// 64 of N = 33, 35 28.1 -> 21.9 ms, 256 of N = 18, 20 14.9 -> 9.9 ms (with one row a
+// warp, its epilogue on every lane, and a slice held whole or not at all).
 // LONG: for groups with a system of M >= kLongRow (a kernel of its own: with both
 // forms in one, the others lost 4-7%).
 template <class T, bool LONG>

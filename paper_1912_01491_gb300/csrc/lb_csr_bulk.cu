@@ -21,12 +21,13 @@
 // by both, one that is zero up to the rounding of t's own terms is kept by
 // neither, and a row with an entry in between goes the general way.
 //
-// What bounds it: the FP64 pipe (k_bulk_rows runs once over the pairs to count
+// What bounds it: the FP64 and the integer pipe (47% and 42% busy) and the loads
+// from the vertices' lists between (k_bulk_rows runs once over the pairs to count
 // and once to fill, 1.0 and 0.65 ms at N = 2000, 1.4 and 1.25 ms with complex
 // products and FP64 comparisons throughout).  Whole assembly, with the scratch
 // kept between calls and the join's passes free of FP64 work for entries that
-// are only counted or dropped: ladder N = 2000 40.9 -> 7.1 ms, N = 1000 12.0 ->
-// 2.0 ms; dimer N = 400 6.2 -> 1.2 ms.
+// are only counted or dropped: ladder N = 2000 40.9 -> 6.5 ms, N = 1000 12.0 ->
+// 2.3 ms; dimer N = 400 6.2 -> 1.2 ms.
 #include <algorithm>
 
 #include "lb_internal.h"

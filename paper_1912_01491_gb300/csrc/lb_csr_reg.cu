@@ -16,9 +16,9 @@
 // its columns and no row pointers, and x is gathered in whole lines.  Entries of
 // a row are summed in CSR order, those of a long row in FP64 by 32 lanes.
 //
-// What bounds it: HBM and its latency at N = 2000 (the ladder's FP32 stage
-// moves 260 MB instead of 416 MB with columns and row pointers: 71 -> 56 us,
-// 4.7 TB/s; FP64 115 -> 107 us, where the FP64 pipe alone takes 82), latency and
+// What bounds it: the latency of HBM at N = 2000 (the ladder's FP32 stage moves
+// 273 MB instead of 408 MB with columns and row pointers: 71 -> 54-57 us, 5.0
+// TB/s; FP64 115 -> 107 us, where the FP64 pipe alone takes 82), latency and
 // the FP64 pipe where the system fits L2 (dimer at N = 400: 35 -> 14 us).
 // Measured slower at N = 2000: chunks of 256 rows staged two ahead by bulk
 // copies (69 us FP32), warps that loop over groups with the next one's loads in

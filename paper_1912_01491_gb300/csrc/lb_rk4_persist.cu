@@ -466,9 +466,10 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_rk4_persist(PersistArgs A
 // 13.9 / 11.4, FP64 N = 30 18.5 / 14.4 (fewer pollers leave L2 to the stores).
 // FP64 rows are a warp's time each: two a warp cost more than they free (N = 40,
 // one stream: 28 / 42), and so do four warps (N = 23 10.5 / 11.9) or eight for eight
-// rows (N = 34 17.9 / 20.8).  Where a launch needs the shared memory of all SMs (FP64
-// N >= 38, FP32 N >= 49) the streams still run one after the other: 8 streams of
-// FP32 N = 50 128 against 119 with a launch per stage, FP64 532 against 389.
+// rows (N = 34 17.9 / 20.8).  Where a launch needs the registers or the shared
+// memory of all SMs (FP64 N >= 33, else N >= 49) the streams still run one after
+// the other: 8 streams of FP32 N = 50 128 against 119 with a launch per stage, FP64
+// 532 against 389.
 int block_warps(int64_t M, int nrows, bool f64) {
   if (M <= 200) return 8;
   if (f64) return nrows <= 7 ? 8 : kMaxWarps;
