@@ -1095,8 +1095,10 @@ cudaError_t assemble_lowrank_csr(const lb::BasisView& B, const double* h, int nP
   const int S = fiber_slices(N);
   // ---- the nonzero pair coefficients of h, and the rows in closed form with the list of the rows that are left.
   // Below 128 levels too many rows are near the diagonal for the extra launches to pay (against the join alone:
-  // ladder N = 70 622 / 567 us, N = 100 638 / 613, N = 140 668 / 688; N = 400 dimer 1.2 / 3.7 ms); more channels than
-  // four have no tables
+  // ladder N = 70 622 / 567 us, N = 100 638 / 613, N = 140 668 / 688; N = 400 dimer 1.2 / 3.7 ms).  The tables hold
+  // 24 N^2 bytes a channel: more than four, or above what the pool hands out (two channels N = 3150, four N = 2290),
+  // and all rows join (five ladders at N = 200 9.4 ms, one 0.65).  Where no row is far from the diagonal the tables
+  // and the count pass are lost, little beside that join (one level coupled to all, N = 128 62.6 ms)
   const bool bulk = N >= 128 && nP <= 4 && csr_bulk_bytes(N, nP) <= kLargeScratch;
   Buf bmem(st), rowc(st), list(st), need(st), bctr(st), hlist(st);  // bctr: join terms, rows left, nonzeros of h
   CsrBulk cb{};
